@@ -254,7 +254,8 @@ def source_key(text):
 
 
 def kernel_hash():
-    return source_key(open(os.path.join(ROOT, "paper_2212_05685_gb300", "csrc", "cheb_kernels.cu")).read())
+    csrc = os.path.join(ROOT, "paper_2212_05685_gb300", "csrc")
+    return source_key("".join(open(os.path.join(csrc, f)).read() for f in ("cheb_kernels.cu", "cheb_march.cuh")))
 
 
 def measured_traffic(name, kernel_key, ldv):

@@ -80,7 +80,8 @@ typedef struct {
                            kpm_observables_noalloc) */
   int32_t block_width;  /* unit start vectors per slab; 0 = as many as fit the
                            context's scratch budget (kpm_set_scratch_budget) */
-  int32_t cols_per_block; /* columns per CTA in the recursion kernel; 0 = default */
+  int32_t cols_per_block; /* columns per CTA in the recursion kernel; 0 = default (FP32 unit
+                           vectors: always 16) */
   double margin;        /* spectral half-width margin of the Gershgorin rescale (0.01) */
   double temperature;   /* 0: T = 0 step and min(eps, 0) in closed form; T > 0: Fermi
                            function 1/(1 + e^{eps/T}) and grand-potential function
@@ -113,9 +114,11 @@ typedef struct {
                            it.  Negative: KPM_EINVAL. */
 } kpm_opts;
 
-/* kpm_opts.flags: run the FP32 recursion two steps per launch where the
- * lattice allows it (default: one step per launch; both give the same bits;
- * kpm_autotune picks the faster) */
+/* kpm_opts.flags: run the FP32 recursion on unit vectors one step more per
+ * launch than by default, where the lattice allows it (default: one step per
+ * launch while the slabs stay in L2 or the budget holds no four slabs, else
+ * two; every choice gives the same bits; kpm_autotune picks the faster).
+ * Launches of several steps need four slabs instead of two. */
 #define KPM_FLAG_DOUBLE_STEP 1
 /* kpm_opts.flags: particle-hole half pass.  Only the N unit columns (j, up)
  * are propagated; the spin-down observables and the other half of the grand

@@ -39,7 +39,7 @@ def _compile(src: str, extra) -> str:
 def build(verbose_ptxas: bool = False, force: bool = False) -> str:
     """Compile every CUDA source for sm_103a and link libkpm.so (in-tree)."""
     os.makedirs(BUILD, exist_ok=True)
-    srcs = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(CSRC, "kpm_internal.cuh"),
+    srcs = [os.path.join(CSRC, s) for s in SOURCES] + [os.path.join(CSRC, "kpm_internal.cuh"), os.path.join(CSRC, "cheb_march.cuh"),
                                                        os.path.join(ROOT, "include", "kpm.h")]
     if not force and os.path.exists(LIB):
         newest = max(os.path.getmtime(s) for s in srcs)

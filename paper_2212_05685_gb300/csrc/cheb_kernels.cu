@@ -36,7 +36,10 @@
 #include <cooperative_groups.h>
 #include <cuda.h>
 
+#include <string.h>
+
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -445,14 +448,7 @@ __device__ __forceinline__ void acc_term(Acc2& a, float2 c, ulonglong2 u) {
 // rows: wm, w0, wp are lattice rows y-1, y, y+1 of a pair-split V in shared
 // memory ([nx][2][NV] float4, already offset by the thread's pair), cf_row the
 // row's 2h~ entries.  Returns the two output rows as (re pair, im pair).
-// SW: rows stored with the two Nambu halves of odd sites swapped (2-column-pair
-// chunks: keeps the 16-byte accesses of a warp's 8-lane phases on distinct banks)
-template <int NV, bool SW = false>
-__device__ __forceinline__ int nambu_slot(int x, int al) {
-  return SW ? (al ^ (x & 1)) : al;
-}
-
-template <int NV, bool SW = false>
+template <int NV>
 __device__ __forceinline__ void stencil_site(const float4* wm, const float4* w0, const float4* wp,
                                              const float2* cf_row, int x, int nx, ulonglong2& o0, ulonglong2& o1) {
   constexpr int RS = 2 * NV;
@@ -460,7 +456,7 @@ __device__ __forceinline__ void stencil_site(const float4* wm, const float4* w0,
   const int xl = x == 0 ? nx - 1 : x - 1;
   const float2* cf = cf_row + x * kCoef;
 #define KPM_L(W, XX, AL) \
-  (*reinterpret_cast<const ulonglong2*>((W) + (XX) * RS + nambu_slot<NV, SW>((XX), (AL)) * NV))
+  (*reinterpret_cast<const ulonglong2*>((W) + (XX) * RS + (AL) * NV))
   Acc2 a0 = {0ull, 0ull, 0ull, 0ull}, a1 = {0ull, 0ull, 0ull, 0ull};
   {
     const float2 d = cf[0];  // (d0, d1): real diagonals of the two Nambu rows
@@ -598,7 +594,7 @@ __device__ __forceinline__ void stencil_2site(const float4* wm, const float4* w0
 
 // moment sums acc[J][s] += a V[K_s(J), J] for the columns of the chunk whose
 // own site lies in lattice row y; wm, w0, wp hold rows y-1, y, y+1
-template <int CB, bool SW = false>
+template <int CB>
 __device__ __forceinline__ void moment_sums(const float4* wm, const float4* w0, const float4* wp, int nx, int y,
                                             int64_t D, const ColMap& cmap, int64_t cb0, int m, double cm, double co,
                                             double2* __restrict__ acc) {
@@ -617,23 +613,9 @@ __device__ __forceinline__ void moment_sums(const float4* wm, const float4* w0, 
     const int dy = kSlotDy[s];
     const float4* w = dy < 0 ? wm : (dy > 0 ? wp : w0);
     const int al = kSlotFlip[s] ? 1 - beta : beta;
-    const float2 val = pair_elem(w + xsl * RS + nambu_slot<NV, SW>(xsl, al) * NV, c);
+    const float2 val = pair_elem(w + xsl * RS + al * NV, c);
     acc_add(acc + J * kSlots + s, s == kSlots - 1 ? co : cm, wgt, (double)val.x, (double)val.y);
     if (s == 0 && cmap.rec) record_diag(cmap, D, m, J, wgt, (double)val.x, (double)val.y);
-  }
-}
-
-// one lattice row of a pair-split V into shared memory with the Nambu halves
-// of odd sites swapped (layout read through nambu_slot<NV, true>)
-template <int NV>
-__device__ __forceinline__ void stage_row_sw(float4* dst, const float4* __restrict__ V, int ly, int nx, int64_t ldq,
-                                             int64_t q0) {
-  const int total = 2 * nx * NV;
-  const float4* base = V + (int64_t)(2 * nx) * ly * ldq + q0;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    const int r = t / NV, c = t - r * NV;
-    const int x = r >> 1, al = r & 1;
-    cp_async16(dst + x * 2 * NV + (al ^ (x & 1)) * NV + c, base + (int64_t)r * ldq + c);
   }
 }
 
@@ -869,11 +851,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // HOOK: the instantiation launched while a failure-path test hook is armed
 // (kpm_inject_lost_copy): its waits read the test's limit and one CTA may
 // skip a window copy; the production instantiation has neither.
-// PR = false: the instantiation for the unit start vectors of a full pass
-// (no probing colours, no half-pass column shift), whose moment sums compile
-// without those branches; probing and half passes run PR = true.  The results
-// are the same bits either way (same items, same arithmetic).
-template <int CB, int MODE, bool HOOK = false, bool PR = true>
+template <int CB, int MODE, bool HOOK = false>
 __device__ __forceinline__ void f32_step_body_tma(const CUtensorMap* tm, int nx, int ny, int64_t D, int64_t ldv,
                                                   int ylen, int brows, const float2* __restrict__ table,
                                                   const float4* Vprev, float4* Vout, ColMap cmap,
@@ -920,14 +898,13 @@ __device__ __forceinline__ void f32_step_body_tma(const CUtensorMap* tm, int nx,
 
   int yj_lo = ny, yj_hi = -1;
   {
-    const int js = PR ? cmap.js : 0;
-    const int64_t clo = cmap.s0 + cb0, chi = min(D >> js, cmap.s0 + cb0 + CB) - 1;
-    if (PR && cmap.probe_p) {
+    const int64_t clo = cmap.s0 + cb0, chi = min(D >> cmap.js, cmap.s0 + cb0 + CB) - 1;
+    if (cmap.probe_p) {
       yj_lo = 0;
       yj_hi = ny - 1;
     } else if (chi >= clo) {
-      yj_lo = (int)(((clo << js) >> 1) / nx);
-      yj_hi = (int)(((chi << js) >> 1) / nx);
+      yj_lo = (int)(((clo << cmap.js) >> 1) / nx);
+      yj_hi = (int)(((chi << cmap.js) >> 1) / nx);
     }
   }
 
@@ -1061,16 +1038,8 @@ __device__ __forceinline__ void f32_step_body_tma(const CUtensorMap* tm, int nx,
       *reinterpret_cast<ulonglong2*>(g + ldq) = o1;
     }
 
-    if (MODE == 1 && acc != nullptr && y >= yj_lo && y <= yj_hi) {
-      // PR = false: unit vectors of the full pass only (the probing items and
-      // the half-pass column shift compiled out)
-      ColMap cu = cmap;
-      if (!PR) {
-        cu.probe_p = 0;
-        cu.js = 0;
-      }
-      moment_sums<CB>(wm - v, w0 - v, wp - v, nx, y, D, cu, cb0, m, am[m], ao[m], acc);
-    }
+    if (MODE == 1 && acc != nullptr && y >= yj_lo && y <= yj_hi)
+      moment_sums<CB>(wm - v, w0 - v, wp - v, nx, y, D, cmap, cb0, m, am[m], ao[m], acc);
     __syncwarp();
     if (lane == 0) mbar_arrive(dbar(q));
     rot = rot_next;
@@ -1094,220 +1063,16 @@ __device__ __forceinline__ void f32_step_body_tma(const CUtensorMap* tm, int nx,
   }
 }
 
-template <int CB, int MODE, bool HOOK = false, bool PR = true>
+template <int CB, int MODE, bool HOOK = false>
 __global__ void __launch_bounds__(512, 1)
     cheb_step_f32_tma_kernel(const __grid_constant__ CUtensorMap tm, int nx, int ny, int64_t D, int64_t ldv,
                              int ylen, int brows, const float2* __restrict__ table, const float4* Vprev, float4* Vout,
                              ColMap cmap, double2* __restrict__ acc, const double* __restrict__ am,
                              const double* __restrict__ ao, int m) {
-  f32_step_body_tma<CB, MODE, HOOK, PR>(&tm, nx, ny, D, ldv, ylen, brows, table, Vprev, Vout, cmap, acc, am, ao, m);
+  f32_step_body_tma<CB, MODE, HOOK>(&tm, nx, ny, D, ldv, ylen, brows, table, Vprev, Vout, cmap, acc, am, ao, m);
 }
 
-// Batched TMA step: blockIdx.z selects the cell; the two slab tensor maps of
-// cell z live in global memory, maps[2 z] over A and maps[2 z + 1] over B;
-// V_m is A at even m and B at odd m (first step: A -> B), in place otherwise
-template <int CB, int MODE>
-__global__ void __launch_bounds__(512, 1)
-    cheb_step_f32_tma_batched_kernel(const CUtensorMap* __restrict__ maps, int nx, int ny, int64_t D, int64_t ldv,
-                                     int ylen, int brows, BatchPtrs b, int m) {
-  const int z = blockIdx.z;
-  const bool cur_b = MODE == 1 && (m & 1);
-  float4* out = reinterpret_cast<float4*>(cur_b ? b.A[z] : b.B[z]);
-  f32_step_body_tma<CB, MODE>(maps + 2 * z + (cur_b ? 1 : 0), nx, ny, D, ldv, ylen, brows,
-                              reinterpret_cast<const float2*>(b.table[z]), out, out,
-                              ColMap{0, 0, 0, 0u, nullptr, nullptr}, b.acc[z], b.am[z], b.ao[z], m);
-}
-
-// FP32 double step: two recursion steps per launch (Eq. alpha applied twice),
-// from V_{m-1} (Vprev) and V_m (Vcur) to V_{m+1} (Vout1) and V_{m+2} (Vout2),
-// all four slabs distinct.  Per pair of steps the slabs are streamed once
-// (read V_{m-1}, V_m, write V_{m+1}, V_{m+2}: 4 x 8 B per row-column instead
-// of 6 x 8 B for two single steps).  The CTA marches a front f from y0-1 to
-// y1 over its band [y0, y1): at each f it computes V_{m+1}[f] from the V_m
-// window (rows f-1..f+1) into a 3-row shared ring, then V_{m+2}[f-1] from the
-// ring (rows f-2..f) and V_m[f-1]; the halo rows y0-1 and y1 of V_{m+1} are
-// computed by every band that needs them and not stored.  Moment sums: a_m V_m
-// at own row f, a_{m+1} V_{m+1} at own row f-1.  Shared memory: V_m ring of
-// 5 rows (3 in use, 2 in flight), V_{m+1} ring of 3 rows, coefficient ring of
-// 4 rows (f-1 and f in use, 2 in flight); two block barriers per front row.
-// Arithmetic is that of two single steps, so results agree bit for bit.
-template <int CB>
-__device__ __forceinline__ void f32_step2_body(int nx, int ny, int64_t D, int64_t ldv, int ylen,
-                                               const float2* __restrict__ table, const float4* __restrict__ Vprev,
-                                               const float4* __restrict__ Vcur, float4* __restrict__ Vout1,
-                                               float4* __restrict__ Vout2, ColMap cmap,
-                                               double2* __restrict__ acc, const double* __restrict__ am,
-                                               const double* __restrict__ ao, int m) {
-  constexpr int NV = CB / 2;
-  constexpr int RS = 2 * NV;
-  constexpr bool SW = NV == 4;  // 8-column chunks: swap the Nambu halves of odd sites
-  const int64_t ldq = ldv / 2;
-
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4* win = reinterpret_cast<float4*>(smem_raw);              // [5][nx][2][NV]  V_m
-  float4* ring = win + 5 * nx * RS;                               // [3][nx][2][NV]  V_{m+1}
-  float2* coef = reinterpret_cast<float2*>(ring + 3 * nx * RS);   // [4][nx][kCoef]
-  const int rowsz = nx * RS;
-  const int crow = nx * kCoef;
-
-  const int64_t cb0 = (int64_t)blockIdx.y * CB;
-  const int64_t q0 = cb0 / 2;
-  const int y0 = blockIdx.x * ylen;
-  const int y1 = min(ny, y0 + ylen);
-  const int nrow = y1 - y0;
-
-  const int v = threadIdx.x % NV;
-  const int xs = threadIdx.x / NV;
-  const int xstep = blockDim.x / NV;
-  const bool own0 = xs < nx, own1 = xs + xstep < nx;
-
-  int yj_lo = ny, yj_hi = -1;
-  {
-    const int64_t clo = cmap.s0 + cb0, chi = min(D >> cmap.js, cmap.s0 + cb0 + CB) - 1;
-    if (cmap.probe_p) {  // every lattice row holds sources of every colour class
-      yj_lo = 0;
-      yj_hi = ny - 1;
-    } else if (chi >= clo) {
-      yj_lo = (int)(((clo << cmap.js) >> 1) / nx);
-      yj_hi = (int)(((chi << cmap.js) >> 1) / nx);
-    }
-  }
-  auto stage_v = [&](float4* dst, int ly) {
-    if (SW)
-      stage_row_sw<NV>(dst, Vcur, ly, nx, ldq, q0);
-    else
-      stage_row<float4, NV>(dst, Vcur, ly, nx, ldq, q0);
-  };
-
-  // V_m row r lives in window slot (r - y0 + 2) % 5, its coefficients in slot
-  // (r - y0 + 2) % 4, V_{m+1} row r in ring slot (r - y0 + 1) % 3.  Prologue
-  // groups: {V rows y0-2..y0, coef y0-2, y0-1}, {V row y0+1, coef y0}; front
-  // step i commits {V row f+3, coef f+2} right after its first barrier.
-  for (int q = 0; q < 3; ++q) stage_v(win + q * rowsz, wrapi(y0 - 2 + q, ny));
-  stage_coef<float2>(coef, table, wrapi(y0 - 2, ny), nx);
-  stage_coef<float2>(coef + crow, table, wrapi(y0 - 1, ny), nx);
-  cp_commit();
-  stage_v(win + 3 * rowsz, wrapi(y0 + 1, ny));
-  stage_coef<float2>(coef + 2 * crow, table, y0, nx);
-  cp_commit();
-
-  ulonglong2 pc[2][2], pn[2][2];
-  const ulonglong2 zero2 = make_ulonglong2(0ull, 0ull);
-  auto load_prev = [&](int y, ulonglong2 (&dst)[2][2]) {
-    const float4* g = Vprev + (2 * ((int64_t)y * nx + xs)) * ldq + q0 + v;
-    const int64_t gstep = 2 * (int64_t)xstep * ldq;
-    dst[0][0] = own0 ? *reinterpret_cast<const ulonglong2*>(g) : zero2;
-    dst[0][1] = own0 ? *reinterpret_cast<const ulonglong2*>(g + ldq) : zero2;
-    dst[1][0] = own1 ? *reinterpret_cast<const ulonglong2*>(g + gstep) : zero2;
-    dst[1][1] = own1 ? *reinterpret_cast<const ulonglong2*>(g + gstep + ldq) : zero2;
-  };
-  load_prev(wrapi(y0 - 1, ny), pc);
-
-  const int nfront = nrow + 2;
-  for (int i = 0; i < nfront; ++i) {
-    const int f = y0 - 1 + i;          // front row (unwrapped)
-    const int fw = wrapi(f, ny);
-    if (i + 1 < nfront) load_prev(wrapi(f + 1, ny), pn);
-    cp_wait_1();
-    __syncthreads();
-    const int s5 = i % 5, s3 = i % 3, s4 = i % 4;
-    // refill the slots of V_m row f-2 and coefficient row f-2 (last read at front f-1)
-    {
-      const int w5 = s5 == 0 ? 4 : s5 - 1;
-      const int w4 = s4 == 0 ? 3 : s4 - 1;
-      if (f + 3 <= y1 + 1) stage_v(win + w5 * rowsz, wrapi(f + 3, ny));
-      if (f + 2 <= y1) stage_coef<float2>(coef + w4 * crow, table, wrapi(f + 2, ny), nx);
-      cp_commit();
-    }
-    const float4* wm = win + s5 * rowsz + v;                            // V_m row f-1
-    const float4* w0 = win + (s5 + 1 == 5 ? 0 : s5 + 1) * rowsz + v;     // f
-    const float4* wp = win + (s5 + 2 >= 5 ? s5 - 3 : s5 + 2) * rowsz + v;  // f+1
-    float4* rf = ring + s3 * rowsz + v;                                  // V_{m+1} row f
-
-    // phase A: V_{m+1}[f] = 2h~ V_m[f] - V_{m-1}[f]
-    {
-      const float2* cf_row = coef + (s4 + 1 == 4 ? 0 : s4 + 1) * crow;  // row f
-      const bool store = f >= y0 && f < y1;
-#pragma unroll
-      for (int it = 0; it < 2; ++it) {
-        if (!(it == 0 ? own0 : own1)) continue;
-        const int x = xs + it * xstep;
-        ulonglong2 o0, o1;
-        stencil_site<NV, SW>(wm, w0, wp, cf_row, x, nx, o0, o1);
-        o0.x = f2sub(o0.x, pc[it][0].x);
-        o0.y = f2sub(o0.y, pc[it][0].y);
-        o1.x = f2sub(o1.x, pc[it][1].x);
-        o1.y = f2sub(o1.y, pc[it][1].y);
-        *reinterpret_cast<ulonglong2*>(rf + x * RS + nambu_slot<NV, SW>(x, 0) * NV) = o0;
-        *reinterpret_cast<ulonglong2*>(rf + x * RS + nambu_slot<NV, SW>(x, 1) * NV) = o1;
-        if (store) {
-          float4* g = Vout1 + (2 * ((int64_t)fw * nx + x)) * ldq + q0 + v;
-          *reinterpret_cast<ulonglong2*>(g) = o0;
-          *reinterpret_cast<ulonglong2*>(g + ldq) = o1;
-        }
-      }
-      if (acc != nullptr && f >= y0 && f < y1 && f >= yj_lo && f <= yj_hi)
-        moment_sums<CB, SW>(wm - v, w0 - v, wp - v, nx, f, D, cmap, cb0, m, am[m], ao[m], acc);
-    }
-    __syncthreads();
-
-    // phase B: V_{m+2}[f-1] = 2h~ V_{m+1}[f-1] - V_m[f-1]
-    if (i >= 2) {
-      const int g = f - 1;
-      const float4* rm = ring + (s3 + 1 == 3 ? 0 : s3 + 1) * rowsz + v;     // V_{m+1} row f-2
-      const float4* r0 = ring + (s3 + 2 >= 3 ? s3 - 1 : s3 + 2) * rowsz + v;  // f-1
-      const float2* cf_row = coef + s4 * crow;                             // row f-1
-#pragma unroll
-      for (int it = 0; it < 2; ++it) {
-        if (!(it == 0 ? own0 : own1)) continue;
-        const int x = xs + it * xstep;
-        ulonglong2 o0, o1;
-        stencil_site<NV, SW>(rm, r0, rf, cf_row, x, nx, o0, o1);
-        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(wm + x * RS + nambu_slot<NV, SW>(x, 0) * NV);
-        const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(wm + x * RS + nambu_slot<NV, SW>(x, 1) * NV);
-        o0.x = f2sub(o0.x, b0.x);
-        o0.y = f2sub(o0.y, b0.y);
-        o1.x = f2sub(o1.x, b1.x);
-        o1.y = f2sub(o1.y, b1.y);
-        float4* gp = Vout2 + (2 * ((int64_t)g * nx + x)) * ldq + q0 + v;
-        *reinterpret_cast<ulonglong2*>(gp) = o0;
-        *reinterpret_cast<ulonglong2*>(gp + ldq) = o1;
-      }
-      if (acc != nullptr && g >= yj_lo && g <= yj_hi)
-        moment_sums<CB, SW>(rm - v, r0 - v, rf - v, nx, g, D, cmap, cb0, m + 1, am[m + 1], ao[m + 1], acc);
-    }
-    pc[0][0] = pn[0][0];
-    pc[0][1] = pn[0][1];
-    pc[1][0] = pn[1][0];
-    pc[1][1] = pn[1][1];
-  }
-  cp_wait_0();
-}
-
-template <int CB>
-__global__ void __launch_bounds__(512, 1)
-    cheb_step2_f32_kernel(int nx, int ny, int64_t D, int64_t ldv, int ylen, const float2* __restrict__ table,
-                          const float4* __restrict__ Vprev, const float4* __restrict__ Vcur, float4* __restrict__ Vout1,
-                          float4* __restrict__ Vout2, ColMap cmap, double2* __restrict__ acc,
-                          const double* __restrict__ am, const double* __restrict__ ao, int m) {
-  f32_step2_body<CB>(nx, ny, D, ldv, ylen, table, Vprev, Vcur, Vout1, Vout2, cmap, acc, am, ao, m);
-}
-
-// Batched step: cells of one shape, blockIdx.z selects the cell; every cell
-// is one full-width slab (s0 = 0).
-template <int CB, int MODE>
-__global__ void __launch_bounds__(512, 1) cheb_step_f32_batched_kernel(int nx, int ny, int64_t D, int64_t ldv,
-                                                                        int ylen, BatchPtrs b, int m) {
-  const int z = blockIdx.z;
-  const float4* cur = reinterpret_cast<const float4*>((m & 1) ? b.B[z] : b.A[z]);
-  float4* out = reinterpret_cast<float4*>((m & 1) ? b.A[z] : b.B[z]);
-  if (MODE == 0) {
-    cur = reinterpret_cast<const float4*>(b.A[z]);
-    out = reinterpret_cast<float4*>(b.B[z]);
-  }
-  f32_step_body<CB, MODE>(nx, ny, D, ldv, ylen, reinterpret_cast<const float2*>(b.table[z]), cur, out, out,
-                          ColMap{0, 0, 0, 0u, nullptr, nullptr}, b.acc[z], b.am[z], b.ao[z], m);
-}
+#include "cheb_march.cuh"
 
 // V0: entry (K, c) of the start vector held by slab column c (unit vector
 // e_{(s0+c) << js}, or probing vector r_{s0+c}); zero in padding columns
@@ -1688,28 +1453,6 @@ size_t smem_f32(int nx) {  // V_m window ring of 5 rows + coefficient ring of 3 
   return sizeof(float4) * (size_t)5 * nx * CB + sizeof(float2) * (size_t)3 * nx * kCoef;
 }
 template <int CB>
-size_t smem_f32x2(int nx) {  // V_m ring of 5 rows + V_{m+1} ring of 3 rows + coefficient ring of 4 rows
-  return sizeof(float4) * (size_t)8 * nx * CB + sizeof(float2) * (size_t)4 * nx * kCoef;
-}
-size_t smem_f32x2_of(int cb, int nx) {
-  return cb == 16 ? smem_f32x2<16>(nx) : cb == 8 ? smem_f32x2<8>(nx) : cb == 4 ? smem_f32x2<4>(nx) : smem_f32x2<2>(nx);
-}
-template <int CB>
-cudaError_t set_smem_f32x2() {
-  return cudaFuncSetAttribute(cheb_step2_f32_kernel<CB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-}
-template <int CB>
-cudaError_t launch_f32x2(const ChebPlan& p, const void* table, const void* Vprev, const void* Vcur, void* Vout1,
-                         void* Vout2, int64_t s0, double2* acc, const double* am, const double* ao, int m,
-                         cudaStream_t s) {
-  const dim3 grid((p.ny + p.ylen2 - 1) / p.ylen2, (unsigned)(p.ldv / CB));
-  cheb_step2_f32_kernel<CB><<<grid, p.nthreads, p.smem2, s>>>(
-      p.nx, p.ny, p.D, p.ldv, p.ylen2, (const float2*)table, (const float4*)Vprev, (const float4*)Vcur,
-      (float4*)Vout1, (float4*)Vout2, colmap(p, s0), acc, am, ao, m);
-  return cudaGetLastError();
-}
-
-template <int CB>
 size_t smem_f64(int nx) {  // V_m window + V_{m-1} rows + coefficient rows
   return sizeof(double2) * ((size_t)6 * 2 * nx * CB + (size_t)2 * nx * kCoef);
 }
@@ -1724,9 +1467,7 @@ cudaError_t set_smem_f32(int nx) {
   if (e != cudaSuccess || CB < 8) return e;
   constexpr int CT = CB >= 8 ? CB : 8;
   for (auto fn : {cheb_step_f32_tma_kernel<CT, 0, false>, cheb_step_f32_tma_kernel<CT, 1, false>,
-                  cheb_step_f32_tma_kernel<CT, 0, true>, cheb_step_f32_tma_kernel<CT, 1, true>,
-                  cheb_step_f32_tma_kernel<CT, 0, false, false>, cheb_step_f32_tma_kernel<CT, 1, false, false>,
-                  cheb_step_f32_tma_kernel<CT, 0, true, false>, cheb_step_f32_tma_kernel<CT, 1, true, false>}) {
+                  cheb_step_f32_tma_kernel<CT, 0, true>, cheb_step_f32_tma_kernel<CT, 1, true>}) {
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e != cudaSuccess) return e;
   }
@@ -1766,24 +1507,6 @@ cudaError_t encode_slab_map(CUtensorMap* tm, const void* V, int64_t D, int64_t l
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 template <int CB>
-cudaError_t set_smem_f32_batched(int nx) {
-  cudaError_t e = cudaFuncSetAttribute(cheb_step_f32_batched_kernel<CB, 0>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(cheb_step_f32_batched_kernel<CB, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kSmemLimit);
-}
-template <int CB>
-cudaError_t launch_f32_batched(const ChebPlan& p, int ncell, const BatchPtrs& b, int m, int mode, cudaStream_t s) {
-  const dim3 grid((p.ny + p.ylen - 1) / p.ylen, (unsigned)(p.ldv / CB), (unsigned)ncell);
-  if (mode == 0)
-    cheb_step_f32_batched_kernel<CB, 0><<<grid, p.nthreads, p.smem, s>>>(p.nx, p.ny, p.D, p.ldv, p.ylen, b, m);
-  else
-    cheb_step_f32_batched_kernel<CB, 1><<<grid, p.nthreads, p.smem, s>>>(p.nx, p.ny, p.D, p.ldv, p.ylen, b, m);
-  return cudaGetLastError();
-}
-
-template <int CB>
 cudaError_t set_smem_f64(int nx) {
   cudaError_t e = cudaFuncSetAttribute(cheb_step_kernel<double, CB, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kSmemLimit);
@@ -1803,17 +1526,9 @@ cudaError_t launch_f32(const ChebPlan& p, const void* table, const void* Vcur, c
     if (e != cudaSuccess) return e;
     const size_t sm = p.smem + kTmaBarBytes;
     // the failure-path test instantiation only while a test hook is armed
-    // and, for the unit start vectors of a full pass, the instantiation
-    // without the probing items and the half-pass shift
-    auto fn = p.probe_p > 0 || p.js != 0
-                  ? (g_step_hook_armed ? (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, true>
-                                                    : cheb_step_f32_tma_kernel<CT, 1, true>)
-                                       : (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, false>
-                                                    : cheb_step_f32_tma_kernel<CT, 1, false>))
-                  : (g_step_hook_armed ? (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, true, false>
-                                                    : cheb_step_f32_tma_kernel<CT, 1, true, false>)
-                                       : (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, false, false>
-                                                    : cheb_step_f32_tma_kernel<CT, 1, false, false>));
+    auto fn = g_step_hook_armed ? (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, true> : cheb_step_f32_tma_kernel<CT, 1, true>)
+                                : (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, false>
+                                             : cheb_step_f32_tma_kernel<CT, 1, false>);
     fn<<<grid, p.nthreads, sm, s>>>(tm, p.nx, p.ny, p.D, p.ldv, p.ylen, p.tma_rows, (const float2*)table,
                                     (const float4*)Vprev, (float4*)Vout, colmap(p, s0), acc, am, ao, m);
     return cudaGetLastError();
@@ -1869,11 +1584,160 @@ cudaError_t launch_f64(const ChebPlan& p, const void* table, const void* Vcur, c
 
 }  // namespace
 
-// Wave model of a one-step launch: chunks x nb CTAs (nb bands of ceil(ny/nb)
-// rows) run one per SM (512 threads at 128 registers) in ceil(CTAs / SMs)
-// waves; a CTA costs its rows plus two halo rows of V_m (one of the three
-// vectors a row streams).  Returns the band heights of the cheapest choices.
-int band_rows_candidates(int ny, int64_t chunks, int* out, int maxn) {
+namespace {
+template <int NV, int NS>
+cudaError_t set_smem_march() {
+  for (auto fn : {cheb_march_kernel<NV, NS, false, false>, cheb_march_kernel<NV, NS, true, false>,
+                  cheb_march_kernel<NV, NS, false, true>, cheb_march_kernel<NV, NS, true, true>}) {
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+template <int NV, int NS>
+void march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, const MarchMaps& pr, const MarchArgs& a,
+                  const ColMap& cm, bool first, cudaStream_t s) {
+  // the failure-path test instantiation only while a test hook is armed
+  auto fn = g_step_hook_armed ? (first ? cheb_march_kernel<NV, NS, true, true> : cheb_march_kernel<NV, NS, false, true>)
+                              : (first ? cheb_march_kernel<NV, NS, true, false> : cheb_march_kernel<NV, NS, false, false>);
+  fn<<<grid, mp.warps * 32, mp.smem, s>>>(v, pr, a, cm);
+}
+}  // namespace
+
+namespace {
+// band heights of a march launch: as many CTAs per SM as registers and shared memory
+// take; a CTA's start (barriers, first copies) costs about five rows, and a launch of
+// several steps computes two more rows for every step but the last
+int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
+  const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>(16 / p.warps, (int64_t)(228 * 1024) / (int64_t)(p.smem + 1024)));
+  return band_rows_candidates(ny, ldv / (2 * kMarchPairs) * p.ntile, out, maxn, per_sm * kSMs, 5.0 + 2.0 * (p.ns - 1));
+}
+
+// Geometry of a march launch: the whole lattice row per CTA where its threads
+// fit, else the fewest equal tiles; then the deepest rings that fit shared
+// memory (several steps: eight rows each), and the band height of the wave model.
+MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows) {
+  MarchPlan p;
+  constexpr int nv = kMarchPairs;
+  auto warps = [&](int tx, bool full) {
+    int n = 2;  // the producer and the moment sums
+    for (int s = 0; s < ns; ++s) n += ((full ? nx : tx + 2 * (ns - 1 - s)) * nv + 31) / 32;
+    return n;
+  };
+  if (warps(nx, true) * 32 <= kMarchThreads) {
+    p.full = 1;
+    p.ntile = 1;
+    p.tx = nx;
+  } else {
+    for (int nt = 2; nt <= nx; ++nt) {
+      const int tx = (nx + nt - 1) / nt;
+      const int last = nx - (nt - 1) * tx;
+      if (warps(tx, false) * 32 <= kMarchThreads && last >= ns && tx >= ns) {
+        p.ntile = nt;
+        p.tx = tx;
+        break;
+      }
+    }
+    if (p.ntile == 0) return p;
+  }
+  p.warps = warps(p.tx, p.full);
+  p.wrow = p.full ? nx : p.tx + 2 * ns;
+  p.crowb = (p.wrow * 208 + 127) / 128 * 128;
+  // a set of rows is issued once the last stage has finished the row `lag` before it;
+  // single step: row i + 2 of V_m then takes the place of one that the stage and the
+  // sums have done with in a ring of lag + 2 rows
+  for (int lag = 8; lag >= (ns == 1 ? 3 : 8); --lag) {
+    p.lag = lag;
+    p.rv = ns == 1 ? lag + 2 : kMarchRows;
+    p.rp = p.rc = ns == 1 ? lag : kMarchRows;
+    p.rs = kMarchRows;
+    p.smem = 32 * (size_t)nv * p.wrow * (p.rv + p.rp + (ns - 1) * p.rs) + (size_t)p.crowb * p.rc +
+             8 * (size_t)kMarchBars * (1 + ns) + 16;
+    if (p.smem <= kSmemLimit) {
+      p.ns = ns;
+      break;
+    }
+  }
+  if (p.ns == 0) return p;
+  int best = ny;
+  march_bands(p, ny, ldv, &best, 1);
+  p.ylen = band_rows > 0 ? std::min(band_rows, ny) : best;
+  return p;
+}
+}  // namespace
+
+namespace {
+cudaError_t march_prepare(const MarchPlan& mp) {
+  return mp.ns == 1 ? set_smem_march<kMarchPairs, 1>()
+                    : mp.ns == 2 ? set_smem_march<kMarchPairs, 2>() : set_smem_march<kMarchPairs, 3>();
+}
+}  // namespace
+
+cudaError_t encode_slab_maps(const ChebPlan& p, const MarchPlan& mp, const void* V, SlabMaps* out, bool as_v,
+                             bool as_p) {
+  static_assert(sizeof(MarchMaps) == 3 * 128 && sizeof(SlabMaps::v) == sizeof(MarchMaps), "SlabMaps layout");
+  auto encode = [&](unsigned char* to, int halo) {  // boxes of a tile with `halo` sites on each side
+    const int sites[3] = {mp.full ? mp.tx : mp.tx + 2 * halo, mp.full ? mp.tx : mp.tx + halo, std::max(1, halo)};
+    for (int k = 0; k < (mp.full ? 1 : 3); ++k) {
+      CUtensorMap t;
+      const cudaError_t e = encode_slab_map(&t, V, p.D, p.ldv, 2 * kMarchPairs, 2 * sites[k]);
+      if (e != cudaSuccess) return e;
+      memcpy(to + 128 * k, &t, 128);
+    }
+    return cudaSuccess;
+  };
+  cudaError_t e = cudaSuccess;
+  if (as_v) e = encode(out->v, mp.ns);
+  if (as_p && e == cudaSuccess) e = encode(out->p, mp.ns - 1);
+  return e;
+}
+
+size_t march_table_bytes(const MarchPlan& mp, int ny) { return (size_t)mp.crowb * ny * mp.ntile; }
+
+cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* table, const SlabMaps& cur,
+                         const SlabMaps& prev, void* outa, void* outb, int64_t s0, double2* acc, const double* am,
+                         const double* ao, int m, bool first, cudaStream_t s) {
+  MarchArgs a;
+  a.nx = p.nx;
+  a.ny = p.ny;
+  a.D = p.D;
+  a.ldq = p.ldv / 2;
+  a.tx = mp.tx;
+  a.ntile = mp.ntile;
+  a.full = mp.full;
+  a.ylen = mp.ylen;
+  a.wrow = mp.wrow;
+  a.lag = mp.lag;
+  a.rp = mp.rp;
+  a.rv = mp.rv;
+  a.rs = mp.rs;
+  a.rc = mp.rc;
+  a.rowb = mp.wrow * 32 * kMarchPairs;
+  a.crowb = mp.crowb;
+  a.table = (const float4*)table;
+  a.outa = (float4*)outa;
+  a.outb = (float4*)outb;
+  a.acc = acc;
+  a.am = am;
+  a.ao = ao;
+  a.m = m;
+  a.grow = 16 * 2 * (int64_t)p.nx * a.ldq;
+  MarchMaps v, pr;
+  memcpy(&v, cur.v, sizeof(v));
+  memcpy(&pr, prev.p, sizeof(pr));
+  const dim3 grid((unsigned)(((p.ny + mp.ylen - 1) / mp.ylen) * mp.ntile), (unsigned)(p.ldv / (2 * kMarchPairs)));
+  const ColMap cm = colmap(p, s0);
+  if (mp.ns == 1) march_launch<kMarchPairs, 1>(mp, grid, v, pr, a, cm, first, s);
+  else if (mp.ns == 2) march_launch<kMarchPairs, 2>(mp, grid, v, pr, a, cm, first, s);
+  else march_launch<kMarchPairs, 3>(mp, grid, v, pr, a, cm, first, s);
+  return cudaGetLastError();
+}
+
+// Wave model of a launch: ctas x nb CTAs (nb bands of ceil(ny/nb) rows) run
+// `slots` at a time in ceil(CTAs / slots) waves; a CTA costs its rows and `extra`
+// more (two halo rows of V_m, one of the three vectors a row streams; for the
+// march kernel its start).  Returns the band heights of the cheapest choices.
+int band_rows_candidates(int ny, int64_t ctas, int* out, int maxn, int slots, double extra) {
   std::vector<std::pair<double, int>> cost;
   int last = -1;
   for (int nb = 1; nb <= ny; ++nb) {
@@ -1881,8 +1745,8 @@ int band_rows_candidates(int ny, int64_t chunks, int* out, int maxn) {
     if (rows == last) continue;
     last = rows;
     const int bands = (ny + rows - 1) / rows;
-    const int64_t waves = (chunks * bands + kSMs - 1) / kSMs;
-    cost.push_back({(double)waves * (rows + 2.0 / 3.0), rows});
+    const int64_t waves = (ctas * bands + slots - 1) / slots;
+    cost.push_back({(double)waves * (rows + extra), rows});
   }
   std::stable_sort(cost.begin(), cost.end(), [](const std::pair<double, int>& a, const std::pair<double, int>& b) {
     return a.first < b.first;
@@ -1892,7 +1756,7 @@ int band_rows_candidates(int ny, int64_t chunks, int* out, int maxn) {
   return n;
 }
 
-ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request, int band_rows) {
+ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request, int band_rows, int steps) {
   ChebPlan p;
   p.nx = nx;
   p.ny = ny;
@@ -1901,6 +1765,13 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
   p.cb = 0;
   p.ldv = 0;
   p.smem = 0;
+  p.tma_rows = 0;
+  p.ylen = ny;
+  p.js = 0;
+  p.probe_p = 0;
+  p.probe_seed = 0;
+  p.xi = nullptr;
+  p.rec = nullptr;
   // widest column chunk that fits shared memory (FP32: 16 columns, FP64: 8);
   // FP32 also needs every thread to own at most two sites of a lattice row
   const int cands32[4] = {16, 8, 4, 2};
@@ -1923,7 +1794,18 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
       break;
     }
   }
-  p.tma_rows = 0;
+  if (precision == KPM_FP32 && steps > 0 && p.cb > 0) {
+    // unit vectors: the march kernel, for every lattice whose row the one-step kernels take
+    p.cb = 2 * kMarchPairs;
+    p.ldv = (width + p.cb - 1) / p.cb * p.cb;
+    p.m1 = plan_march(nx, ny, p.ldv, 1, band_rows);
+    p.mk = steps > 1 ? plan_march(nx, ny, p.ldv, steps, band_rows) : p.m1;
+    if (p.mk.ns == 0) p.mk = p.m1;
+    p.ylen = p.mk.ylen;
+    p.nthreads = 32 * p.mk.warps;
+    p.smem = p.mk.smem;
+    return p;
+  }
   if (precision == KPM_FP32 && p.cb >= 8 && p.smem + kTmaBarBytes <= kSmemLimit) {
     // TMA staging: the 2 Nx Nambu rows of a window row in nb equal boxes of
     // at most 256 rows, each landing on a 128-byte boundary of shared memory
@@ -1935,14 +1817,6 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
       break;
     }
   }
-  p.cb2 = 0;
-  p.ylen2 = 0;
-  p.smem2 = 0;
-  p.js = 0;
-  p.probe_p = 0;
-  p.probe_seed = 0;
-  p.xi = nullptr;
-  p.rec = nullptr;
   if (p.cb == 0) return p;
   p.ldv = (width + p.cb - 1) / p.cb * p.cb;
   // band height of the one-step kernels: the caller's, else the best of the
@@ -1951,48 +1825,31 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
   int best_rows = ny;
   band_rows_candidates(ny, chunks, &best_rows, 1);
   p.ylen = band_rows > 0 ? std::min(band_rows, ny) : best_rows;
-  if (precision == KPM_FP32) {
-    // double step: widest chunk (<= cb) whose three rings fit; bands of at
-    // least 4 rows (each band recomputes two halo rows of V_{m+1} and reads
-    // four halo rows of V_m), about two waves of one CTA per SM
-    for (int k = 0; k < 4; ++k) {
-      const int c2 = cands32[k];
-      if (c2 > p.cb || nx > 2 * (p.nthreads / (c2 / 2))) continue;
-      const size_t sm2 = smem_f32x2_of(c2, nx);
-      if (sm2 > kSmemLimit) continue;
-      const int64_t ch2 = p.ldv / c2;
-      const int yb2 = (int)std::min<int64_t>(ny, std::max<int64_t>(1, (2 * kSMs + ch2 - 1) / ch2));
-      const int yl2 = (ny + yb2 - 1) / yb2;
-      if (yl2 >= 4) {
-        p.cb2 = c2;
-        p.ylen2 = yl2;
-        p.smem2 = sm2;
-        break;
-      }
-    }
-  }
   return p;
+}
+
+
+// Two steps per launch where the slabs stream from memory and the tile fills its
+// warps: 100x100 (13 or 14 stage warps) 1248 against 1457 us per step, a 2500-column
+// slab of it 180 against 213; 64x64, whose tiles of 22 sites fill 11.5, 275 against 266
+int march_steps(int nx, int ny, int64_t width) {
+  const int64_t D = 2 * (int64_t)nx * ny;
+  if (16 * D * width <= kMarchL2) return 1;
+  const MarchPlan p = plan_march(nx, ny, width, 2, 0);
+  return p.ns == 2 && p.warps >= 15 ? 2 : 1;
+}
+
+int plan_band_candidates(const ChebPlan& p, int* out, int maxn) {
+  if (p.mk.ns) return march_bands(p.mk, p.ny, p.ldv, out, maxn);
+  return band_rows_candidates(p.ny, p.ldv / p.cb, out, maxn);
 }
 
 size_t table_bytes_per_site(int precision) { return (size_t)kCoef * (precision == KPM_FP32 ? 8 : 16); }
 
-cudaError_t launch_cheb_step2(const ChebPlan& p, const void* table, const void* Vprev, const void* Vcur,
-                              void* Vout1, void* Vout2, int64_t s0, double2* acc, const double* am,
-                              const double* ao, int m, cudaStream_t s) {
-  switch (p.cb2) {
-    case 16: return launch_f32x2<16>(p, table, Vprev, Vcur, Vout1, Vout2, s0, acc, am, ao, m, s);
-    case 8: return launch_f32x2<8>(p, table, Vprev, Vcur, Vout1, Vout2, s0, acc, am, ao, m, s);
-    case 4: return launch_f32x2<4>(p, table, Vprev, Vcur, Vout1, Vout2, s0, acc, am, ao, m, s);
-    case 2: return launch_f32x2<2>(p, table, Vprev, Vcur, Vout1, Vout2, s0, acc, am, ao, m, s);
-  }
-  return cudaErrorInvalidValue;
-}
-
 cudaError_t cheb_prepare(const ChebPlan& p, int precision) {
-  if (precision == KPM_FP32 && p.cb2 > 0) {
-    cudaError_t e = p.cb2 == 16 ? set_smem_f32x2<16>() : p.cb2 == 8 ? set_smem_f32x2<8>()
-                  : p.cb2 == 4 ? set_smem_f32x2<4>() : set_smem_f32x2<2>();
-    if (e != cudaSuccess) return e;
+  if (p.mk.ns) {
+    const cudaError_t e = march_prepare(p.mk);
+    return e != cudaSuccess ? e : march_prepare(p.m1);
   }
   if (precision == KPM_FP32) {
     switch (p.cb) {
@@ -2040,6 +1897,13 @@ cudaError_t launch_cheb_step(const ChebPlan& p, int precision, const void* table
                              int64_t s0, double2* acc, const double* am, const double* ao, int m, int mode,
                              cudaStream_t s, const void* Vprev) {
   if (!Vprev) Vprev = Vout;
+  if (precision == KPM_FP32 && p.m1.ns) {
+    SlabMaps cur, prev;
+    cudaError_t e = encode_slab_maps(p, p.m1, Vcur, &cur, true, false);
+    if (e == cudaSuccess) e = encode_slab_maps(p, p.m1, Vprev, &prev, false, true);
+    if (e != cudaSuccess) return e;
+    return launch_march(p, p.m1, table, cur, prev, nullptr, Vout, s0, acc, am, ao, m, mode == 0, s);
+  }
   if (precision == KPM_FP32) {
     switch (p.cb) {
       case 16: return launch_f32<16>(p, table, Vcur, Vprev, Vout, s0, acc, am, ao, m, mode, s);
@@ -2061,61 +1925,6 @@ cudaError_t launch_cheb_step(const ChebPlan& p, int precision, const void* table
       case 2: return launch_f64<2>(p, table, Vcur, Vprev, Vout, s0, acc, am, ao, m, mode, s);
       case 1: return launch_f64<1>(p, table, Vcur, Vprev, Vout, s0, acc, am, ao, m, mode, s);
     }
-  }
-  return cudaErrorInvalidValue;
-}
-
-template <int CB>
-cudaError_t set_smem_f32_tma_batched() {
-  cudaError_t e = cudaFuncSetAttribute(cheb_step_f32_tma_batched_kernel<CB, 0>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(cheb_step_f32_tma_batched_kernel<CB, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kSmemLimit);
-}
-
-cudaError_t cheb_prepare_batched(const ChebPlan& p) {
-  if (p.tma_rows > 0) {
-    const cudaError_t e = p.cb == 16 ? set_smem_f32_tma_batched<16>() : set_smem_f32_tma_batched<8>();
-    if (e != cudaSuccess) return e;
-  }
-  switch (p.cb) {
-    case 16: return set_smem_f32_batched<16>(p.nx);
-    case 8: return set_smem_f32_batched<8>(p.nx);
-    case 4: return set_smem_f32_batched<4>(p.nx);
-    case 2: return set_smem_f32_batched<2>(p.nx);
-  }
-  return cudaErrorInvalidValue;
-}
-
-size_t batch_maps_bytes(int ncell) { return (size_t)2 * ncell * sizeof(CUtensorMap); }
-
-cudaError_t encode_batch_maps(const ChebPlan& p, int ncell, const BatchPtrs& b, void* host_maps) {
-  CUtensorMap* out = static_cast<CUtensorMap*>(host_maps);
-  for (int z = 0; z < ncell; ++z) {
-    cudaError_t e = encode_slab_map(out + 2 * z, b.A[z], p.D, p.ldv, p.cb, p.tma_rows);
-    if (e == cudaSuccess) e = encode_slab_map(out + 2 * z + 1, b.B[z], p.D, p.ldv, p.cb, p.tma_rows);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-cudaError_t launch_cheb_step_batched(const ChebPlan& p, int ncell, const BatchPtrs& b, int m, int mode,
-                                     cudaStream_t s, const void* maps) {
-  if (maps != nullptr && p.tma_rows > 0 && (p.cb == 16 || p.cb == 8)) {
-    const dim3 grid((p.ny + p.ylen - 1) / p.ylen, (unsigned)(p.ldv / p.cb), (unsigned)ncell);
-    const size_t sm = p.smem + kTmaBarBytes;
-    const CUtensorMap* tm = static_cast<const CUtensorMap*>(maps);
-    auto fn = p.cb == 16 ? (mode == 0 ? cheb_step_f32_tma_batched_kernel<16, 0> : cheb_step_f32_tma_batched_kernel<16, 1>)
-                         : (mode == 0 ? cheb_step_f32_tma_batched_kernel<8, 0> : cheb_step_f32_tma_batched_kernel<8, 1>);
-    fn<<<grid, p.nthreads, sm, s>>>(tm, p.nx, p.ny, p.D, p.ldv, p.ylen, p.tma_rows, b, m);
-    return cudaGetLastError();
-  }
-  switch (p.cb) {
-    case 16: return launch_f32_batched<16>(p, ncell, b, m, mode, s);
-    case 8: return launch_f32_batched<8>(p, ncell, b, m, mode, s);
-    case 4: return launch_f32_batched<4>(p, ncell, b, m, mode, s);
-    case 2: return launch_f32_batched<2>(p, ncell, b, m, mode, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -26,7 +26,7 @@ struct kpm_ctx {
   uint64_t budget = 24ull << 30;
 
   // scratch (owned)
-  void* slab[4] = {nullptr, nullptr, nullptr, nullptr};  // two, or four for the double-step recursion
+  void* slab[4] = {nullptr, nullptr, nullptr, nullptr};  // two, or four for several steps per launch
   int slab_n = 0;
   size_t slab_bytes = 0;
   double2* xi = nullptr;  // probing phases conj(xi_J) of the current pass
@@ -99,7 +99,6 @@ struct kpm_ctx {
   size_t bhost_n = 0;
   cudaGraphExec_t bgraph = nullptr;
   std::vector<char> bkey;
-  std::vector<void*> bmaps;        // per shape class: device copy of its cells' slab tensor maps
   // persistent recursion of the batch: cell table, work items (longest first),
   // item counter; events around its launch
   void* pbuf = nullptr;
@@ -211,7 +210,7 @@ struct PassPlan {
   ChebPlan cheb;
   int64_t width;  // unit columns per slab
   size_t elem;    // bytes per complex
-  bool dbl;       // FP32 double-step recursion (four slabs)
+  bool deeper;    // FP32: a step more per launch than by default (KPM_FLAG_DOUBLE_STEP)
   int64_t c0, c1; // pass columns [c0, c1) (all: 0, pass_columns)
   int sb, se;     // sites whose observables the pass writes (all: 0, N)
   bool ranged;    // a proper sub-range of the sites
@@ -225,7 +224,8 @@ int64_t balanced_width(int64_t D, int64_t width) {
   return (D + n - 1) / n;
 }
 
-int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp) {
+// single: FP32 unit vectors one step per launch (a caller that needs every vector)
+int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp, bool single = false) {
   if (!o) return fail(ctx, KPM_EINVAL, "opts is null");
   if (o->M < 1) return fail(ctx, KPM_EINVAL, "M must be >= 1");
   if (o->precision != KPM_FP32 && o->precision != KPM_FP64 && o->precision != KPM_DF64)
@@ -254,32 +254,40 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp)
     if (pp->ranged && (o->flags & KPM_FLAG_PH_HALF))
       return fail(ctx, KPM_EINVAL, "KPM_FLAG_PH_HALF and a site range do not combine");
   }
-  const bool want_dbl = o->precision == KPM_FP32 && (o->flags & KPM_FLAG_DOUBLE_STEP) && pp_ == 0;
+  const bool march = o->precision == KPM_FP32 && pp_ == 0;  // FP32 unit vectors
+  const bool deeper = march && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
   const int js = (o->flags & KPM_FLAG_PH_HALF) ? 1 : 0;
   // start vectors of the pass: unit columns (those of the site range), or R = 2 p^2 probing vectors
   pp->c0 = pp->ranged ? 2 * (int64_t)pp->sb : 0;
   pp->c1 = pp->ranged ? 2 * (int64_t)pp->se : (pp_ > 0 ? std::min<int64_t>(D, 2 * (int64_t)pp_ * pp_) : (D >> js));
   const int64_t ncols = pp->c1 - pp->c0;
-  int64_t width = o->block_width > 0 ? std::min<int64_t>(o->block_width, ncols) : ncols;
-  if (o->block_width == 0) {
-    const int64_t fit = (int64_t)(ctx->budget / ((want_dbl ? 4 : 2) * (uint64_t)D * pp->elem));
-    width = balanced_width(ncols, std::min<int64_t>(width, std::max<int64_t>(fit, 1)));
-  }
-  pp->cheb = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows);
+  // slab width: as asked, else as many columns as fit the budget; several steps per
+  // launch need four slabs, a default that does not fit them takes one step
+  auto width_of = [&](int slabs) {
+    if (o->block_width > 0) return std::min<int64_t>(o->block_width, ncols);
+    const int64_t fit = (int64_t)(ctx->budget / ((uint64_t)slabs * (uint64_t)D * pp->elem));
+    return balanced_width(ncols, std::min<int64_t>(ncols, std::max<int64_t>(fit, 1)));
+  };
+  int64_t width = width_of(2);
+  int steps = march ? (single ? 1 : march_steps(m->nx, m->ny, width)) : 0;
+  if (steps > 1 && (o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
+  if (deeper) ++steps;
+  if (steps > 1) width = width_of(4);
+  pp->cheb = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows, steps);
+  pp->deeper = deeper && pp->cheb.mk.ns == steps;
   pp->cheb.js = js;
   pp->cheb.probe_p = pp_;
   pp->cheb.probe_seed = (uint32_t)o->probe_seed;
   if (pp->cheb.cb == 0) return fail(ctx, KPM_EINVAL, "lattice row too wide for the shared-memory window");
   // slabs advance by the padded width: every unit column belongs to exactly one slab
   pp->width = pp->cheb.ldv;
-  pp->dbl = want_dbl && pp->cheb.cb2 > 0;
   return KPM_OK;
 }
 
 int ensure_pass_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, const PassPlan& pp) {
   const int64_t D = pp.cheb.D;
   const size_t slab = (size_t)D * pp.cheb.ldv * pp.elem;
-  const int nslab = pp.dbl ? 4 : 2;
+  const int nslab = pp.cheb.mk.ns > 1 ? 4 : 2;
   int r;
   if (ctx->slab_bytes < slab || ctx->slab_n < nslab) {
     drop_graph(ctx);
@@ -305,7 +313,9 @@ int ensure_pass_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, con
     if (ctx->xi_bytes < (size_t)D * sizeof(double2)) drop_graph(ctx);
     if ((r = ensure(ctx, &ctx->xi, &ctx->xi_bytes, (size_t)D * sizeof(double2)))) return r;
   }
-  const size_t tb = (size_t)m->nx * m->ny * table_bytes_per_site(o->precision);
+  // FP32 unit vectors: the entries in the ring rows' layout of both launch plans
+  const size_t tb = pp.cheb.mk.ns ? march_table_bytes(pp.cheb.mk, m->ny) + march_table_bytes(pp.cheb.m1, m->ny)
+                                  : (size_t)m->nx * m->ny * table_bytes_per_site(o->precision);
   if (ctx->table_bytes < tb) drop_graph(ctx);
   if ((r = ensure(ctx, &ctx->table, &ctx->table_bytes, tb))) return r;
   if (ctx->coef_n < (size_t)o->M) {
@@ -354,19 +364,67 @@ int enqueue_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, const Pass
   double nb = 0.0;
   const double vec = (double)p.D * (double)p.ldv * (double)pp.elem;  // bytes of one slab vector
   KPM_CU(launch_coefficients(M, ab, ctx->am, ctx->ao, s, p.js, o->temperature));
-  if (prec == KPM_FP32)
+  SlabMaps mk[4], m1[4];
+  char* const table1 = static_cast<char*>(ctx->table) + (p.mk.ns > 1 ? march_table_bytes(p.mk, p.ny) : 0);
+  if (p.mk.ns) {
+    if (p.mk.ns > 1) {
+      KPM_CU(launch_march_table(*m, p.mk, fields, ab, (float4*)ctx->table, s));
+      for (int k = 0; k < 4; ++k) KPM_CU(encode_slab_maps(p, p.mk, ctx->slab[k], &mk[k]));
+      nl += 1;
+    }
+    KPM_CU(launch_march_table(*m, p.m1, fields, ab, (float4*)table1, s));
+    for (int k = 0; k < (p.mk.ns > 1 ? 4 : 2); ++k) KPM_CU(encode_slab_maps(p, p.m1, ctx->slab[k], &m1[k]));
+  } else if (prec == KPM_FP32)
     KPM_CU(launch_scale_table_f32(*m, fields, ab, (float2*)ctx->table, s));
   else if (prec == KPM_DF64)
     KPM_CU(launch_scale_table_df(*m, fields, ab, (float4*)ctx->table, s));
   else
     KPM_CU(launch_scale_table_f64(*m, fields, ab, (double2*)ctx->table, s));
   nl += 2;
-  for (int64_t s0 = pp.c0; s0 < pp.c1; s0 += pp.width) {
-    // X0 = V_{mm-1}, X1 = V_mm; Y0, Y1 the free pair of the double-step recursion
-    void* X0 = ctx->slab[0];
-    void* X1 = ctx->slab[1];
-    void* Y0 = pp.dbl ? ctx->slab[2] : nullptr;
-    void* Y1 = pp.dbl ? ctx->slab[3] : nullptr;
+  for (int64_t s0 = pp.c0; p.mk.ns && s0 < pp.c1; s0 += pp.width) {
+    // ix, iy: the slabs of V_{mm-1} and V_mm
+    int ix = 0, iy = 0, mm = 0;  // highest vector computed so far
+    KPM_CU(launch_cheb_init(p, prec, ctx->slab[0], s0, ctx->acc, ctx->am, ctx->ao, s));
+    nl += 1;
+    if (events && s0 == pp.c0) KPM_CU(cudaEventRecordWithFlags(ctx->ev[0], s, cudaEventRecordExternal));
+    while (mm < M - 1) {
+      const bool first = mm == 0;
+      if (p.mk.ns > 1 && mm + p.mk.ns <= M - 1) {
+        int ia = 0, ib;
+        while (ia == ix || ia == iy) ++ia;
+        for (ib = ia + 1; ib == ix || ib == iy; ++ib) {}
+        KPM_CU(launch_march(p, p.mk, ctx->table, mk[iy], mk[ix], ctx->slab[ia], ctx->slab[ib], s0, ctx->acc, ctx->am,
+                            ctx->ao, mm, first, s));
+        nb += (first ? 3 : 4) * vec;
+        ix = ia;
+        iy = ib;
+        mm += p.mk.ns;
+      } else {
+        // one step, in place over V_{mm-1} (the first into the second slab)
+        const int io = first ? 1 : ix;
+        KPM_CU(launch_march(p, p.m1, table1, m1[iy], m1[ix], nullptr, ctx->slab[io], s0, ctx->acc, ctx->am,
+                            ctx->ao, mm, first, s));
+        nb += (first ? 2 : 3) * vec;
+        ix = iy;
+        iy = io;
+        mm += 1;
+      }
+      nr += 1;
+    }
+    if (events && s0 + pp.width >= pp.c1) KPM_CU(cudaEventRecordWithFlags(ctx->ev[1], s, cudaEventRecordExternal));
+    if (M >= 2) {
+      KPM_CU(launch_cheb_gather(p, prec, ctx->slab[iy], s0, ctx->acc, ctx->am, ctx->ao, M - 1, s));
+      nl += 1;
+      if (tail) {  // alpha_{M-2}, alpha_{M-1} of this slab for a later backward pass
+        char* t = static_cast<char*>(tail) + (size_t)(2 * ((s0 - pp.c0) / pp.width)) * (size_t)vec;
+        KPM_CU(cudaMemcpyAsync(t, ctx->slab[ix], (size_t)vec, cudaMemcpyDeviceToDevice, s));
+        KPM_CU(cudaMemcpyAsync(t + (size_t)vec, ctx->slab[iy], (size_t)vec, cudaMemcpyDeviceToDevice, s));
+      }
+    }
+  }
+  for (int64_t s0 = pp.c0; !p.mk.ns && s0 < pp.c1; s0 += pp.width) {
+    void* X0 = ctx->slab[0];  // V_{mm-1}
+    void* X1 = ctx->slab[1];  // V_mm
     KPM_CU(launch_cheb_init(p, prec, X0, s0, ctx->acc, ctx->am, ctx->ao, s));
     nl += 1;
     if (events && s0 == pp.c0) KPM_CU(cudaEventRecordWithFlags(ctx->ev[0], s, cudaEventRecordExternal));
@@ -376,15 +434,6 @@ int enqueue_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, const Pass
       nb += 2 * vec;
     }
     int mm = 1;  // highest vector index computed so far
-    if (pp.dbl) {
-      for (; mm + 2 <= M - 1; mm += 2) {
-        KPM_CU(launch_cheb_step2(p, ctx->table, X0, X1, Y0, Y1, s0, ctx->acc, ctx->am, ctx->ao, mm, s));
-        nr += 1;
-        nb += 4 * vec;
-        std::swap(X0, Y0);
-        std::swap(X1, Y1);
-      }
-    }
     for (; mm + 1 <= M - 1; ++mm) {
       // V_{mm+1} = 2 h~ V_mm - V_{mm-1} in place over V_{mm-1}
       KPM_CU(launch_cheb_step(p, prec, ctx->table, X1, X0, s0, ctx->acc, ctx->am, ctx->ao, mm, 1, s));
@@ -519,7 +568,6 @@ int kpm_destroy(kpm_ctx* ctx) {
   if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
   for (auto& c : ctx->cells)
     if (c.mem) cudaFree(c.mem);
-  for (void* p : ctx->bmaps) cudaFree(p);
   if (ctx->pbuf) cudaFree(ctx->pbuf);
   for (cudaEvent_t e : ctx->pev)
     if (e) cudaEventDestroy(e);
@@ -934,7 +982,7 @@ int kpm_backward(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
     o.block_width = (int)balanced_width(ncol, std::max<int64_t>(1, std::min<int64_t>(ncol, fit)));
   }
   PassPlan pp;
-  if ((r = plan_pass(ctx, model, &o, &pp))) return r;
+  if ((r = plan_pass(ctx, model, &o, &pp, true))) return r;
   if ((r = ensure_pass_scratch(ctx, model, &o, pp))) return r;
   const ChebPlan& p = pp.cheb;
   const size_t vbytes = (size_t)D * p.ldv * elem;
@@ -964,7 +1012,7 @@ int kpm_backward(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
   void* B = ctx->slab[1];
   KPM_CU(launch_coefficients(M, ab, ctx->am, ctx->ao, s, 0, o.temperature));
   if (prec == KPM_FP32)
-    KPM_CU(launch_scale_table_f32(*model, fields, ab, (float2*)ctx->table, s));
+    KPM_CU(launch_march_table(*model, p.m1, fields, ab, (float4*)ctx->table, s));
   else
     KPM_CU(launch_scale_table_f64(*model, fields, ab, (double2*)ctx->table, s));
   // seeds of the columns outside the site range are zero: their backward
@@ -1173,14 +1221,9 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   for (size_t k = 0; k < members.size(); ++k) {
     const kpm_model& m0 = models[members[k][0]];
     const int64_t D = 2 * (int64_t)m0.nx * m0.ny;
-    plans[k] = plan_cheb(m0.nx, m0.ny, D, prec, opts->cols_per_block, opts->band_rows);
+    plans[k] = plan_cheb(m0.nx, m0.ny, D, prec, opts->cols_per_block, opts->band_rows, 1);
     if (plans[k].cb == 0) return fail(ctx, KPM_EINVAL, "lattice row too wide for the shared-memory window");
-    // spread one step over the whole batch: y bands so that every cell fills its share
-    const int64_t chunks = plans[k].ldv / plans[k].cb;
-    const int64_t want = std::max<int64_t>(1, 4 * 152 / (int64_t)std::max<size_t>(1, members[k].size()));
-    const int yb = (int)std::min<int64_t>(m0.ny, std::max<int64_t>(1, (want + chunks - 1) / chunks));
-    plans[k].ylen = std::max(1, (m0.ny + yb - 1) / yb);
-    cudaError_t e = prec == KPM_FP32 ? cheb_prepare_batched(plans[k]) : cheb_prepare(plans[k], prec);
+    cudaError_t e = cheb_prepare(plans[k], prec);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "prepare");
   }
 
@@ -1211,6 +1254,10 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
 
   // per-cell scratch, one allocation per cell
   auto al = [](size_t n) { return (n + 255) & ~(size_t)255; };
+  auto tab_bytes = [&](int k, int N) {
+    return prec == KPM_FP32 && !persist[k] ? march_table_bytes(plans[k].m1, plans[k].ny)
+                                           : (size_t)N * table_bytes_per_site(prec);
+  };
   bool realloc = (int)ctx->cells.size() != ncell;
   std::vector<size_t> need(ncell);
   for (int c = 0; c < ncell; ++c) {
@@ -1219,7 +1266,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     const int k = cls_of[std::make_pair(models[c].nx, models[c].ny)];
     // (cells of the persistent recursion keep their vectors in shared memory: no slabs)
     need[c] = al(26 * (size_t)N * 8) * 2 + al((size_t)M * 8) * 2 + al(16 * 8) + al((size_t)D * kSlots * 16) +
-              al((size_t)N * table_bytes_per_site(prec)) + (persist[k] ? 0 : 2 * al((size_t)D * plans[k].ldv * elem));
+              al(tab_bytes(k, N)) + (persist[k] ? 0 : 2 * al((size_t)D * plans[k].ldv * elem));
     if (!realloc && ctx->cells[c].bytes < need[c]) realloc = true;
   }
   if (realloc) {
@@ -1250,7 +1297,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     C.ao = (double*)b; b += al((size_t)M * 8);
     C.misc = (double*)b; b += al(16 * 8);
     C.acc = (double2*)b; b += al((size_t)D * kSlots * 16);
-    C.table = b; b += al((size_t)N * table_bytes_per_site(prec));
+    C.table = b; b += al(tab_bytes(k, N));
     if (persist[k]) {
       C.A = C.B = nullptr;
     } else {
@@ -1305,43 +1352,6 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
     ctx->bgraph = nullptr;
     cudaStream_t c0 = ctx->cap;
-    // per shape class: the cells' pointers and, for the TMA-staged step, the
-    // tensor maps of their slabs, uploaded before the capture (the graph
-    // reads them from device memory on every replay)
-    std::vector<BatchPtrs> bps(members.size());
-    std::vector<const void*> maps_of(members.size(), nullptr);
-    for (size_t k = 0; k < members.size(); ++k) {
-      BatchPtrs& bp = bps[k];
-      memset(&bp, 0, sizeof(bp));
-      for (size_t z = 0; z < members[k].size(); ++z) {
-        kpm_ctx::Cell& C = ctx->cells[members[k][z]];
-        bp.A[z] = C.A;
-        bp.B[z] = C.B;
-        bp.table[z] = C.table;
-        bp.acc[z] = C.acc;
-        bp.am[z] = C.am;
-        bp.ao[z] = C.ao;
-      }
-    }
-    if (prec == KPM_FP32) {
-      while (ctx->bmaps.size() < members.size()) {
-        void* d = nullptr;
-        if (cudaMalloc(&d, batch_maps_bytes(kMaxBatch)) != cudaSuccess) {
-          cudaGetLastError();
-          return fail(ctx, KPM_ENOMEM, "cudaMalloc of the batch tensor maps failed");
-        }
-        ctx->bmaps.push_back(d);
-      }
-      KPM_CU(cudaStreamSynchronize(c0));  // no replay of an older graph still reads the maps
-      for (size_t k = 0; k < members.size(); ++k) {
-        if (plans[k].tma_rows == 0 || persist[k]) continue;
-        const int nz = (int)members[k].size();
-        std::vector<CUtensorMap> host((size_t)2 * nz);
-        KPM_CU(encode_batch_maps(plans[k], nz, bps[k], host.data()));
-        KPM_CU(cudaMemcpy(ctx->bmaps[k], host.data(), batch_maps_bytes(nz), cudaMemcpyHostToDevice));
-        maps_of[k] = ctx->bmaps[k];
-      }
-    }
     // persistent recursion: the cell table and the work items, longest first
     // (an item's time grows with its cell's band, nx ceil(ny / kPClu) sites),
     // uploaded before the capture like the tensor maps
@@ -1412,8 +1422,10 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
       KPM_TRY(launch_shift_eps(N, C.fields, mu_eff + c, C.misc + 6, C.misc + 2, ctx->bred, c0));
       KPM_TRY(launch_gershgorin(m, C.fields, opts->margin, C.misc, ctx->bred, c0));
       KPM_TRY(launch_coefficients(M, C.misc, C.am, C.ao, c0, 0, opts->temperature));
-      if (prec == KPM_FP32)
+      if (prec == KPM_FP32 && persist[C.cls])
         KPM_TRY(launch_scale_table_f32(m, C.fields, C.misc, (float2*)C.table, c0));
+      else if (prec == KPM_FP32)
+        KPM_TRY(launch_march_table(m, p.m1, C.fields, C.misc, (float4*)C.table, c0));
       else
         KPM_TRY(launch_scale_table_f64(m, C.fields, C.misc, (double2*)C.table, c0));
       if (!persist[C.cls]) KPM_TRY(launch_cheb_init(p, prec, C.A, 0, C.acc, C.am, C.ao, c0));
@@ -1425,19 +1437,13 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
       cudaStream_t sk = ctx->fork[k];
       KPM_TRY(cudaStreamWaitEvent(sk, ctx->join_ev, 0));
       const ChebPlan& p = plans[k];
-      if (prec == KPM_FP32) {
-        const int nz = (int)members[k].size();
-        KPM_TRY(launch_cheb_step_batched(p, nz, bps[k], 0, 0, sk, maps_of[k]));
-        for (int mm = 1; mm <= M - 2; ++mm) KPM_TRY(launch_cheb_step_batched(p, nz, bps[k], mm, 1, sk, maps_of[k]));
-      } else {
-        for (size_t z = 0; z < members[k].size(); ++z) {
-          kpm_ctx::Cell& C = ctx->cells[members[k][z]];
-          KPM_TRY(launch_cheb_step(p, prec, C.table, C.A, C.B, 0, C.acc, C.am, C.ao, 0, 0, sk));
-          for (int mm = 1; mm <= M - 2; ++mm) {
-            const void* cur = (mm & 1) ? C.B : C.A;
-            void* out = (mm & 1) ? C.A : C.B;
-            KPM_TRY(launch_cheb_step(p, prec, C.table, cur, out, 0, C.acc, C.am, C.ao, mm, 1, sk));
-          }
+      for (size_t z = 0; z < members[k].size(); ++z) {
+        kpm_ctx::Cell& C = ctx->cells[members[k][z]];
+        KPM_TRY(launch_cheb_step(p, prec, C.table, C.A, C.B, 0, C.acc, C.am, C.ao, 0, 0, sk));
+        for (int mm = 1; mm <= M - 2; ++mm) {
+          const void* cur = (mm & 1) ? C.B : C.A;
+          void* out = (mm & 1) ? C.A : C.B;
+          KPM_TRY(launch_cheb_step(p, prec, C.table, cur, out, 0, C.acc, C.am, C.ao, mm, 1, sk));
         }
       }
       KPM_TRY(cudaEventRecord(ctx->fork_ev[k], sk));
@@ -1582,15 +1588,14 @@ int kpm_autotune(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
       PassPlan pp;
       if (plan_pass(ctx, model, &o, &pp) != KPM_OK) continue;
       if (pp.cheb.cb != c) continue;  // chunk does not fit for this lattice
-      if (mode && !pp.dbl) continue;  // no double-step plan for this lattice
-      // band heights of the one-step kernels: the default (the wave model's
-      // best), its next two, and one band per chunk (the double-step kernel
-      // keeps its own bands)
+      if (mode && !pp.deeper) continue;  // no deeper plan for this lattice
+      // band heights: the default (the wave model's best), its next two, and one
+      // band per chunk (the deeper launches: the default)
       int bands[4] = {0, 0, 0, 0};
       int nband = 1;
       if (!mode) {
         int cand[4];
-        int nc = band_rows_candidates(model->ny, pp.cheb.ldv / pp.cheb.cb, cand, 3);
+        int nc = plan_band_candidates(pp.cheb, cand, 3);
         cand[nc++] = model->ny;
         for (int k = 0; k < nc; ++k) {
           bool seen = cand[k] == pp.cheb.ylen;

@@ -14,8 +14,25 @@ constexpr int kSlots = 10;     // accumulated entries per unit column (9 local r
 constexpr int kCoef = 26;      // complex 2h~ entries per site (both Nambu rows, padded)
 constexpr int kRedBlock = 256; // threads of the reduction kernels
 
+// Launch geometry of the FP32 march kernel (ns recursion steps per launch).
+struct MarchPlan {
+  int ns = 0;                  // steps per launch (0: not planned)
+  int tx = 0, ntile = 0, full = 0;  // sites per tile, tiles per lattice row, one tile covers the row
+  int ylen = 0;                // lattice rows per band
+  int wrow = 0, crowb = 0;     // sites of a ring row, bytes of its entries
+  int lag = 0, rp = 0, rv = 0, rs = 0, rc = 0;  // rows of the rings (plan_march)
+  int warps = 0;
+  size_t smem = 0;
+};
+// tensor maps of one slab as V_m and as V_{m-1} of a launch (three CUtensorMap each)
+struct alignas(64) SlabMaps {
+  unsigned char v[3 * 128], p[3 * 128];
+};
+
 // Launch geometry of the recursion kernel (shared with the host planner).
 struct ChebPlan {
+  MarchPlan mk;    // FP32 unit vectors: the pass's launches of several steps (or one)
+  MarchPlan m1;    // and the single step
   int nx, ny;
   int64_t D;       // 2 N
   int64_t ldv;     // slab width padded to a multiple of cb (complex elements per row)
@@ -23,11 +40,7 @@ struct ChebPlan {
   int ylen;        // lattice rows marched per CTA
   int nthreads;
   size_t smem;     // dynamic shared memory per CTA
-  int tma_rows;    // FP32 step: Nambu rows per TMA box of a window row (0: cp.async staging)
-  // FP32 double-step kernel (two recursion steps per launch); cb2 = 0: not used
-  int cb2;         // columns per CTA (divides cb)
-  int ylen2;       // lattice rows per band
-  size_t smem2;
+  int tma_rows;    // FP32 probing step: Nambu rows per TMA box of a window row (0: cp.async staging)
   // slab column c holds unit vector J = (s0 + c) << js (js = 1: particle-hole
   // half pass over the columns (j, up) only; the pass covers D >> js columns)
   int js;
@@ -54,16 +67,7 @@ inline int64_t pass_columns(const ChebPlan& p) {
   return p.probe_p > 0 ? 2 * (int64_t)p.probe_p * p.probe_p : (p.D >> p.js);
 }
 
-// Per-cell pointers of a batch of equally shaped cells (FP32 recursion).
-constexpr int kMaxBatch = 64;
-struct BatchPtrs {
-  void* A[kMaxBatch];
-  void* B[kMaxBatch];
-  const void* table[kMaxBatch];
-  double2* acc[kMaxBatch];
-  const double* am[kMaxBatch];
-  const double* ao[kMaxBatch];
-};
+constexpr int kMaxBatch = 64;  // cells of one shape in a batched call (FP32)
 
 // ---------------------------------------------------------------- rmft_kernels.cu
 cudaError_t launch_peierls(const kpm_model& m, double* phi, cudaStream_t s);
@@ -85,6 +89,9 @@ cudaError_t launch_coefficients(int M, const double* ab, double* am, double* ao,
 // per-site table of 2h~ entries in precision T (kCoef complex per site)
 cudaError_t launch_scale_table_f32(const kpm_model& m, const double* fields, const double* ab,
                                    float2* table, cudaStream_t s);
+// the same entries in the order the march kernel reads them, 13 float4 per site, row by row of every tile of the plan
+cudaError_t launch_march_table(const kpm_model& m, const MarchPlan& mp, const double* fields, const double* ab,
+                               float4* table, cudaStream_t s);
 // double-float table: entries as float4 (re_hi, re_lo, im_hi, im_lo)
 cudaError_t launch_scale_table_df(const kpm_model& m, const double* fields, const double* ab, float4* table,
                                   cudaStream_t s);
@@ -117,10 +124,17 @@ cudaError_t launch_update(int N, double* params, double* obs, double* mu_eff, co
 int reduce_scratch_doubles(int64_t n);
 
 // ---------------------------------------------------------------- cheb_kernels.cu
-ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0);
-// up to maxn band heights (lattice rows per CTA) for chunks column chunks of
-// an ny-row lattice, best first by a wave model of the one-step kernels
-int band_rows_candidates(int ny, int64_t chunks, int* out, int maxn);
+// steps: FP32 recursion steps per launch of unit-vector slabs (the march kernel,
+// chunks of 16 columns); 0: the one-step kernels of probing slabs, FP64 and double-float
+ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0, int steps = 0);
+// FP32 steps per launch at which unit-vector slabs of `width` columns run fastest
+int march_steps(int nx, int ny, int64_t width);
+// up to maxn band heights (lattice rows per CTA) for `ctas` CTAs per band of an
+// ny-row lattice, best first by a wave model: `slots` CTAs run at a time, each
+// costing its rows and `extra` more
+int band_rows_candidates(int ny, int64_t ctas, int* out, int maxn, int slots = 152, double extra = 2.0 / 3.0);
+// the same for a plan's launches
+int plan_band_candidates(const ChebPlan& p, int* out, int maxn);
 // bytes of the per-site 2h~ table (kCoef complex entries)
 size_t table_bytes_per_site(int precision);
 cudaError_t cheb_prepare(const ChebPlan& p, int precision);
@@ -133,27 +147,23 @@ cudaError_t launch_cheb_init(const ChebPlan& p, int precision, void* V0, int64_t
 cudaError_t launch_cheb_step(const ChebPlan& p, int precision, const void* table, const void* Vcur,
                              void* Vout, int64_t s0, double2* acc, const double* am,
                              const double* ao, int m, int mode, cudaStream_t s, const void* Vprev = nullptr);
-// FP32 double step: Vout1 = V_{m+1}, Vout2 = V_{m+2} from Vprev = V_{m-1}, Vcur = V_m
-// (four distinct slabs), accumulating a_m V_m and a_{m+1} V_{m+1} unless acc is null
-cudaError_t launch_cheb_step2(const ChebPlan& p, const void* table, const void* Vprev, const void* Vcur,
-                              void* Vout1, void* Vout2, int64_t s0, double2* acc, const double* am,
-                              const double* ao, int m, cudaStream_t s);
-// batched FP32 step over ncell cells of one shape (plan p, full-width slabs);
-// with p.tma_rows > 0 and `maps` (device copy of the 2 ncell tensor maps that
-// encode_batch_maps writes to host memory, batch_maps_bytes(ncell) bytes,
-// 64-byte aligned) the TMA-staged kernel runs, else the cp.async one
-cudaError_t cheb_prepare_batched(const ChebPlan& p);
-size_t batch_maps_bytes(int ncell);
-cudaError_t encode_batch_maps(const ChebPlan& p, int ncell, const BatchPtrs& b, void* host_maps);
-cudaError_t launch_cheb_step_batched(const ChebPlan& p, int ncell, const BatchPtrs& b, int m, int mode,
-                                     cudaStream_t s, const void* maps = nullptr);
-// device fault word of the TMA-staged FP32 step (bit 0: a bounded wait
+// device fault word of the TMA-staged FP32 steps (bit 0: a bounded wait
 // expired; bit 1: shared memory misaligned for TMA); sticky for the process
 cudaError_t read_step_fault(unsigned int* out);
 cudaError_t clear_step_fault();
 // failure-path test hook: the next drop_copies CTAs of the TMA step skip one
 // window copy; bounded-wait limit of later launches (0: the default 2 s)
 cudaError_t set_step_failure_test(int drop_copies, uint64_t wait_limit_ns);
+// FP32 march: tensor maps of a slab, and one launch of mp.ns steps from V_m = Vcur
+// and V_{m-1} = Vprev to V_{m+ns-1} = outa and V_{m+ns} = outb (ns = 1: outb
+// only, in place over Vprev allowed); first: m = 0, V_1 = h~ V_0, no Vprev.
+// acc may be null (no moment sums).
+cudaError_t encode_slab_maps(const ChebPlan& p, const MarchPlan& mp, const void* V, SlabMaps* out, bool as_v = true,
+                             bool as_p = true);
+cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* table, const SlabMaps& cur,
+                         const SlabMaps& prev, void* outa, void* outb, int64_t s0, double2* acc, const double* am,
+                         const double* ao, int m, bool first, cudaStream_t s);
+size_t march_table_bytes(const MarchPlan& mp, int ny);
 // table conj(xi_J) of the probing phases, J < D
 cudaError_t launch_probe_phases(const ChebPlan& p, double2* xi_conj, cudaStream_t s);
 // acc += a_m V[local rows] for the slab's columns (no recursion)

@@ -99,23 +99,31 @@ extern "C" int kpm_observables_noalloc(const kpm_model* m, const kpm_opts* o, co
   const size_t off_ao = align256(off_am + (size_t)o->M * sizeof(double));
   const size_t off_red = align256(off_ao + (size_t)o->M * sizeof(double));
   const size_t off_tab = align256(off_red + (size_t)reduce_scratch_doubles(0) * sizeof(double));
-  const size_t off_acc = align256(off_tab + (size_t)N * table_bytes_per_site(o->precision));
-  const size_t off_slab = align256(off_acc + (size_t)D * kSlots * sizeof(double2));
-  if (off_slab >= kNoAllocScratchBytes) return KPM_EINVAL;  // the lattice or M exceeds the static scratch
-
-  // widest slab (unit columns per recursion) whose two buffers fit the rest
-  const size_t avail = kNoAllocScratchBytes - off_slab;
-  int64_t width = std::min<int64_t>(o->block_width > 0 ? o->block_width : D,
-                                    (int64_t)(avail / (2 * (size_t)D * elem)));
+  // widest slab (unit columns per recursion) whose two buffers fit the rest: FP32 by
+  // the march kernel, or, where its 16-column chunk does not fit, by the narrower
+  // chunks of the one-step kernels
+  size_t off_acc = 0, off_slab = 0;
   ChebPlan p;
-  p.cb = 0;
-  while (width >= 1) {
-    p = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows);
+  int64_t width = 0;
+  for (int steps = o->precision == KPM_FP32 ? 1 : 0; steps >= 0; --steps) {
+    p = plan_cheb(m->nx, m->ny, D, o->precision, o->cols_per_block, o->band_rows, steps);
     if (p.cb == 0) return KPM_EINVAL;
-    if (2 * (size_t)D * p.ldv * elem + 2 * 255 <= avail) break;
-    width -= p.cb;
+    off_acc = align256(off_tab + (p.m1.ns ? march_table_bytes(p.m1, m->ny) : (size_t)N * table_bytes_per_site(o->precision)));
+    off_slab = align256(off_acc + (size_t)D * kSlots * sizeof(double2));
+    if (off_slab >= kNoAllocScratchBytes) {  // the lattice or M exceeds the static scratch
+      width = 0;
+      continue;
+    }
+    const size_t avail = kNoAllocScratchBytes - off_slab;
+    width = std::min<int64_t>(o->block_width > 0 ? o->block_width : D, (int64_t)(avail / (2 * (size_t)D * elem)));
+    while (width >= 1) {
+      p = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows, steps);
+      if (2 * (size_t)D * p.ldv * elem + 2 * 255 <= avail) break;
+      width -= p.cb;
+    }
+    if (width >= 1) break;
   }
-  if (width < 1 || p.cb == 0) return KPM_EINVAL;  // not even one column chunk fits
+  if (width < 1) return KPM_EINVAL;  // not even one column chunk fits
 
   void* base = nullptr;
   cudaError_t e = scratch_address(dev, (cudaStream_t)stream, &base);
@@ -144,7 +152,9 @@ extern "C" int kpm_observables_noalloc(const kpm_model* m, const kpm_opts* o, co
   } while (0)
   KPM_NA(cheb_prepare(p, prec));
   KPM_NA(launch_coefficients(M, ab, am, ao, s, 0, o->temperature));
-  if (prec == KPM_FP32)
+  if (p.m1.ns)
+    KPM_NA(launch_march_table(*m, p.m1, fields, ab, (float4*)table, s));
+  else if (prec == KPM_FP32)
     KPM_NA(launch_scale_table_f32(*m, fields, ab, (float2*)table, s));
   else
     KPM_NA(launch_scale_table_f64(*m, fields, ab, (double2*)table, s));

@@ -476,19 +476,20 @@ __device__ __forceinline__ float4 to_c<float4>(Cplx v) {
 }
 
 
+// the kCoef entries of 2h~ of site i: the two real diagonals (packed), hops of
+// the up and down rows to the neighbours (+1,0) (-1,0) (0,+1) (0,-1) (+1,+1)
+// (-1,-1) (+1,-1) (-1,+1), pairings of both rows to the first four
 template <typename C>
-__global__ void scale_table_kernel(kpm_model m, const double* __restrict__ fld, const double* __restrict__ ab,
-                                   C* __restrict__ table) {
+__device__ __forceinline__ void site_entries(const kpm_model& m, const double* __restrict__ fld,
+                                             const double* __restrict__ ab, int i, C (&out)[kCoef]) {
   const int nx = m.nx, ny = m.ny, N = nx * ny;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
   const Layout L{N};
   const double a = ab[0], b = ab[1];
   const double s = 2.0 / a;
-  C* out = table + (size_t)i * kCoef;
   out[0] = to_c<C>(cx(2.0 * (L.n(fld, 0, i) - b) / a, 2.0 * (-L.n(fld, 1, i) - b) / a));
   // forward bond d for neighbours k = 1,3,5,7 and backward for k = 2,4,6,8
   const int dir_of_k[8] = {0, 0, 1, 1, 2, 2, 3, 3};
+#pragma unroll
   for (int k = 0; k < 8; ++k) {
     const int d = dir_of_k[k];
     Cplx up, dn;
@@ -505,6 +506,7 @@ __global__ void scale_table_kernel(kpm_model m, const double* __restrict__ fld, 
   }
   // nn neighbours k = 1..4 in the order (+1,0) (-1,0) (0,+1) (0,-1) -> e = 0, 2, 1, 3
   const int e_of_k[4] = {0, 2, 1, 3};
+#pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int e = e_of_k[k];
     const int j = shift(i, kNnX[e], kNnY[e], nx, ny);
@@ -512,6 +514,59 @@ __global__ void scale_table_kernel(kpm_model m, const double* __restrict__ fld, 
     out[21 + k] = to_c<C>(cscale(cconj(L.F(fld, (e + 2) & 3, j)), -s));
   }
   out[25] = to_c<C>(cx(0.0, 0.0));
+}
+
+template <typename C>
+__global__ void scale_table_kernel(kpm_model m, const double* __restrict__ fld, const double* __restrict__ ab,
+                                   C* __restrict__ table) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m.nx * m.ny) return;
+  C e[kCoef];
+  site_entries<C>(m, fld, ab, i, e);
+  C* out = table + (size_t)i * kCoef;
+#pragma unroll
+  for (int k = 0; k < kCoef; ++k) out[k] = e[k];
+}
+
+// the entries in the order in which the march kernel's sums use them: for each
+// component the diagonal, then per neighbour its hop and (first four) its pairing
+// (25 floats each, 52 with padding), for the sites of every tile's ring row: halo
+// sites on its left, its own (tx, fewer in the last tile), halo sites on its right
+__global__ void march_table_kernel(kpm_model m, const double* __restrict__ fld, const double* __restrict__ ab,
+                                   float4* __restrict__ table, int tx, int ntile, int wrow, int crow, int halo) {
+  const int at = blockIdx.x * blockDim.x + threadIdx.x;
+  if (at >= m.ny * ntile * wrow) return;
+  const int p = at % wrow, tile = at / wrow % ntile, y = at / wrow / ntile;
+  const int x0 = tile * tx, w = min(m.nx, x0 + tx) - x0;
+  int k = p - halo;            // site x0 + k
+  if (p >= halo + tx) k = w + (p - halo - tx);
+  else if (k >= w) k = w - 1;  // no site: any
+  const int x = (x0 + k + m.nx) % m.nx, i = y * m.nx + x;
+  float2 e[kCoef];
+  site_entries<float2>(m, fld, ab, i, e);
+  float o[2 * kCoef];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const bool up = c == 0;
+    float* q = o + 25 * c;
+    q[0] = up ? e[0].x : e[0].y;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int to = k < 4 ? 1 + 4 * k : 17 + 2 * (k - 4);
+      const float2 hop = up ? e[1 + k] : e[9 + k];
+      q[to] = hop.x;
+      q[to + 1] = hop.y;
+      if (k < 4) {
+        const float2 pair = up ? e[17 + k] : e[21 + k];
+        q[to + 2] = pair.x;
+        q[to + 3] = pair.y;
+      }
+    }
+  }
+  o[50] = o[51] = 0.f;
+  float4* out = table + (size_t)(at / wrow) * crow + p * (kCoef / 2);
+#pragma unroll
+  for (int k = 0; k < kCoef / 2; ++k) out[k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
 }
 
 // Observables from the accumulated entries of F_M(h~) e_J (readings N2, N3):
@@ -1014,6 +1069,14 @@ cudaError_t launch_scale_table_f32(const kpm_model& m, const double* fields, con
                                    cudaStream_t s) {
   const int N = m.nx * m.ny;
   scale_table_kernel<float2><<<(N + 127) / 128, 128, 0, s>>>(m, fields, ab, table);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_march_table(const kpm_model& m, const MarchPlan& mp, const double* fields, const double* ab,
+                               float4* table, cudaStream_t s) {
+  const int n = m.ny * mp.ntile * mp.wrow;
+  march_table_kernel<<<(n + 127) / 128, 128, 0, s>>>(m, fields, ab, table, mp.tx, mp.ntile, mp.wrow,
+                                                      mp.crowb / 16, mp.full ? 0 : mp.ns);
   return cudaGetLastError();
 }
 
