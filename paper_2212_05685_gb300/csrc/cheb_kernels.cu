@@ -19,19 +19,17 @@
 // unevaluated FP32 sum hi + lo, and runs the FP64 kernel's structure with
 // double-float arithmetic.  FP32 stores each column pair (2p, 2p+1) as
 // (re_2p, re_2p+1, im_2p, im_2p+1) so that one packed f32x2 FMA advances two
-// columns.  h~ is a 13-point stencil
-// per row (diagonal, eight hops, four pairings), read from a per-site table
-// of kCoef complex 2h~ entries.
+// columns.  h~ is a 13-point stencil per row (diagonal, eight hops, four
+// pairings), read from a per-site table of kCoef complex 2h~ entries.
 //
-// Each CTA owns a chunk of CB columns and a band of lattice rows y0..y1-1.  It
-// marches along y keeping lattice rows y-1, y, y+1 of V_m (all Nx sites, both
-// Nambu components, CB columns) in shared memory, with the next rows and
-// coefficient rows in flight (FP32 chunks of 8 or 16 columns: TMA tensor and
-// bulk copies completing on mbarriers; otherwise cp.async), so every V_m
-// element is read from global memory once per CTA while serving the 13 rows
-// that need it.
-// V_{m-1} is read ahead (FP32: into registers one row early; FP64: through
-// cp.async) and V_{m+1} written in place with coalesced 16-byte accesses.
+// FP32 runs the march kernel (cheb_march.cuh).  The kernels of this file serve FP64
+// and double-float, and FP32 where the march kernel's 16-column chunk does not
+// fit (the allocation-free call): each CTA owns a chunk of CB columns and a band
+// of lattice rows y0..y1-1 and marches along y keeping lattice rows y-1, y, y+1
+// of V_m (all Nx sites, both Nambu components, CB columns) in shared memory, the
+// next rows and coefficient rows in flight by cp.async, so every V_m element is
+// read from global memory once per CTA while serving the 13 rows that need it;
+// V_{m-1} is read ahead and V_{m+1} written in place.
 // No tensor cores: the stencil is sparse, not a dense contraction.
 #include <cooperative_groups.h>
 #include <cuda.h>
@@ -756,19 +754,11 @@ __global__ void __launch_bounds__(512, 1)
   f32_step_body<CB, MODE>(nx, ny, D, ldv, ylen, table, Vcur, Vprev, Vout, cmap, acc, am, ao, m);
 }
 
-// ---- FP32 step with TMA staging ------------------------------------------
-// Same stencil, ring depths, arithmetic and results as f32_step_body; the
-// V_m window rows and the coefficient rows are moved by the tensor memory
-// accelerator instead of per-thread cp.async: one elected thread issues, per
-// lattice row, a 2-D tensor copy of the row's 2 Nx Nambu rows x CB columns
-// (cp.async.bulk.tensor, one box or a few row boxes) and a 1-D bulk copy of
-// the row's 2h~ entries, each completing on an mbarrier of its ring slot with
-// the byte count expected; every thread waits on the slots it reads.  Slot
-// reuse is ordered by row-done mbarriers instead of a block barrier (see the
-// body).  Waits are bounded in time: a CTA whose copies do not land sets the fault
-// word, waits (bounded) for its copies in flight and writes NaN over its
-// output rows, so a failed launch shows in the observables instead of
-// hanging the device.
+// ---- TMA copies and bounded waits (the march kernel) ----------------------
+// Waits on mbarriers are bounded in time: a CTA whose copies do not land sets the
+// fault word, waits (bounded) for its copies in flight and writes NaN over its
+// output rows, so a failed launch shows in the observables instead of hanging the
+// device.
 __device__ unsigned int g_step_fault;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -816,260 +806,14 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 }
 
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s: orders of magnitude above a lattice row's copies
-// bounded-wait limit of the TMA step (kWaitLimitNs unless a test shortened it)
+// bounded-wait limit of the march kernel (kWaitLimitNs unless a test shortened it)
 // and the number of CTAs that are still to skip one window copy (test hook of
 // the failure path: a skipped copy leaves nothing in flight, so only the
 // waits on its slot run out)
 __device__ unsigned long long g_wait_limit_ns = kWaitLimitNs;
 __device__ int g_drop_copy;
-// wait of the TMA step: the limit (g_wait_limit_ns >> shift) is read only once
-// the first poll has failed, so the fast path carries nothing extra
-__device__ __noinline__ bool step_wait_slow(uint32_t bar, uint32_t parity, int shift) {
-  const uint64_t lim = *reinterpret_cast<volatile unsigned long long*>(&g_wait_limit_ns) >> shift;
-  return mbar_wait_slow(bar, parity, lim);
-}
-template <bool HOOK>
-__device__ __forceinline__ bool step_wait(uint32_t bar, uint32_t parity, int shift = 0) {
-  if (HOOK) return mbar_try(bar, parity) || step_wait_slow(bar, parity, shift);
-  return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, kWaitLimitNs >> shift);
-}
-
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-}
-
-// Rows without a block barrier: the warps run up to two lattice rows apart.
-// Slot reuse is ordered by a third ring of mbarriers, done[r % 3], on which
-// every warp arrives once it has finished row r (count = warps per CTA); the
-// issuing thread waits for done(r - 1) before it refills the slots that row
-// r - 1 was the last to read.  A warp at row r needs window row r + 2, issued
-// only after done(r - 3), so no warp runs more than two rows ahead of the
-// slowest and no mbarrier phase is reused before it has been waited on.
-// Sites of a row: thread (xs, v) takes site xs, and the nx - xstep sites
-// beyond the first round go to xstep-groups in an order rotated from row to
-// row, so that every warp does the same work averaged over a few rows.
-// HOOK: the instantiation launched while a failure-path test hook is armed
-// (kpm_inject_lost_copy): its waits read the test's limit and one CTA may
-// skip a window copy; the production instantiation has neither.
-template <int CB, int MODE, bool HOOK = false>
-__device__ __forceinline__ void f32_step_body_tma(const CUtensorMap* tm, int nx, int ny, int64_t D, int64_t ldv,
-                                                  int ylen, int brows, const float2* __restrict__ table,
-                                                  const float4* Vprev, float4* Vout, ColMap cmap,
-                                                  double2* __restrict__ acc, const double* __restrict__ am,
-                                                  const double* __restrict__ ao, int m) {
-  constexpr int NV = CB / 2;
-  constexpr int RS = 2 * NV;
-  const int64_t ldq = ldv / 2;
-
-  extern __shared__ __align__(1024) unsigned char smem_tma[];
-  float4* win = reinterpret_cast<float4*>(smem_tma);                       // [5][nx][2][NV]
-  float2* coef = reinterpret_cast<float2*>(win + 5 * nx * RS);             // [3][nx][kCoef]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(coef + 3 * nx * kCoef);    // full V 0..4, full coef 5..7, done 8..10
-  volatile int* fail_flag = reinterpret_cast<volatile int*>(bars + 11);
-  const int rowsz = nx * RS;
-  const int crow = nx * kCoef;
-
-  const int64_t cb0 = (int64_t)blockIdx.y * CB;
-  const int64_t q0 = cb0 / 2;
-  const int y0 = blockIdx.x * ylen;
-  const int y1 = min(ny, y0 + ylen);
-  const int nrow = y1 - y0;
-
-  const int v = threadIdx.x % NV;
-  const int xs = threadIdx.x / NV;
-  const int xstep = blockDim.x / NV;
-  const int extra = nx - xstep;  // sites beyond the first round (nx <= 2 xstep, planner)
-  const bool own0 = xs < nx;
-  const int lane = threadIdx.x & 31;
-  // second site of the thread in a row whose extra sites start at xs-group
-  // `rot` (advanced by `rstep` from row to row), or -1
-  const int rstep = extra > 0 ? extra : 0;
-  auto site1 = [&](int rot) {
-    if (extra <= 0) return -1;
-    int d = xs - rot;
-    d = d < 0 ? d + xstep : d;
-    return d < extra ? xstep + d : -1;
-  };
-  auto next_rot = [&](int rot) {
-    rot += rstep;
-    return rot >= xstep ? rot - xstep : rot;
-  };
-  int rot = 0;  // rotation of the CTA's current row
-
-  int yj_lo = ny, yj_hi = -1;
-  {
-    const int64_t clo = cmap.s0 + cb0, chi = min(D >> cmap.js, cmap.s0 + cb0 + CB) - 1;
-    if (cmap.probe_p) {
-      yj_lo = 0;
-      yj_hi = ny - 1;
-    } else if (chi >= clo) {
-      yj_lo = (int)(((clo << cmap.js) >> 1) / nx);
-      yj_hi = (int)(((chi << cmap.js) >> 1) / nx);
-    }
-  }
-
-  const uint32_t bar0 = smem_u32(bars);
-  const uint32_t vbytes = (uint32_t)(2 * nx * CB * 8);  // one window row: 2 Nx Nambu rows x CB complex FP32
-  const uint32_t cbytes = (uint32_t)(nx * kCoef * 8);   // one coefficient row
-  const int nbox = 2 * nx / brows;
-  // window row w holds lattice row y0 - 1 + w (w = 0 .. nrow + 1) in slot w % 5,
-  // coefficient row c holds row y0 + c (c = 0 .. nrow - 1) in slot c % 3
-  int w_hi = -1, c_hi = -1;  // last window / coefficient row issued (issuing thread)
-  auto issue_v = [&](int w) {
-    const int ly = wrapi(y0 - 1 + w, ny);
-    const uint32_t bar = bar0 + 8 * (w % 5);
-    const uint32_t dst = smem_u32(win + (w % 5) * rowsz);
-    if (HOOK && w == 2 && *reinterpret_cast<volatile int*>(&g_drop_copy) > 0 && atomicSub(&g_drop_copy, 1) > 0) {
-      w_hi = w;  // skipped: the slot's phase never completes
-      return;
-    }
-    mbar_expect_tx(bar, vbytes);
-    for (int b = 0; b < nbox; ++b)
-      tma_load_2d(dst + (uint32_t)(b * brows * CB * 8), tm, (int)(2 * cb0), 2 * nx * ly + b * brows, bar);
-    w_hi = w;
-  };
-  auto issue_c = [&](int c) {
-    const uint32_t bar = bar0 + 8 * (5 + c % 3);
-    mbar_expect_tx(bar, cbytes);
-    bulk_load(smem_u32(coef + (c % 3) * crow), table + (int64_t)(y0 + c) * crow, cbytes, bar);
-    c_hi = c;
-  };
-  auto vbar = [&](int w) { return bar0 + 8 * (w % 5); };
-  auto vpar = [&](int w) { return (uint32_t)((w / 5) & 1); };
-  auto cbar = [&](int c) { return bar0 + 8 * (5 + c % 3); };
-  auto cpar = [&](int c) { return (uint32_t)((c / 3) & 1); };
-  auto dbar = [&](int r) { return bar0 + 8 * (8 + r % 3); };
-  auto dpar = [&](int r) { return (uint32_t)((r / 3) & 1); };
-
-  auto poison = [&]() {  // NaN over the CTA's output rows
-    const float nan = __int_as_float(0x7fc00000);
-    const float4 nan4 = make_float4(nan, nan, nan, nan);
-    for (int t = threadIdx.x; t < nrow * 2 * nx * NV; t += blockDim.x) {
-      const int r = t / NV, c = t - r * NV;
-      Vout[((int64_t)2 * nx * y0 + r) * ldq + q0 + c] = nan4;
-    }
-  };
-  // after a fault anywhere, later CTAs and launches only mark their outputs
-  if (*reinterpret_cast<volatile unsigned int*>(&g_step_fault) != 0u) {
-    poison();
-    return;
-  }
-  const bool aligned = (smem_u32(win) & 127u) == 0 && (blockDim.x & 31) == 0;
-  if (aligned && threadIdx.x == 0) {
-    for (int k = 0; k < 8; ++k) mbar_init(bar0 + 8 * k, 1);
-    for (int k = 8; k < 11; ++k) mbar_init(bar0 + 8 * k, blockDim.x >> 5);
-    *fail_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  }
-  if (!__syncthreads_and(aligned)) {
-    if (threadIdx.x == 0) atomicOr(&g_step_fault, 2u);
-    poison();
-    return;
-  }
-  if (threadIdx.x == 0) {
-    for (int w = 0; w <= min(3, nrow + 1); ++w) issue_v(w);
-    for (int c = 0; c <= min(1, nrow - 1); ++c) issue_c(c);
-  }
-
-  ulonglong2 pc[2][2], pn[2][2];
-  const ulonglong2 zero2 = make_ulonglong2(0ull, 0ull);
-  auto load_prev = [&](int y, int r, ulonglong2 (&dst)[2][2]) {
-    const float4* g = Vprev + (2 * ((int64_t)y * nx + xs)) * ldq + q0 + v;
-    dst[0][0] = own0 ? *reinterpret_cast<const ulonglong2*>(g) : zero2;
-    dst[0][1] = own0 ? *reinterpret_cast<const ulonglong2*>(g + ldq) : zero2;
-    const int x1 = site1(r);
-    const float4* g1 = Vprev + (2 * ((int64_t)y * nx + (x1 < 0 ? 0 : x1))) * ldq + q0 + v;
-    dst[1][0] = x1 >= 0 ? *reinterpret_cast<const ulonglong2*>(g1) : zero2;
-    dst[1][1] = x1 >= 0 ? *reinterpret_cast<const ulonglong2*>(g1 + ldq) : zero2;
-  };
-  if (MODE == 1) load_prev(y0, rot, pc);
-
-  const u64 half2 = 0x3F0000003F000000ull;  // (0.5f, 0.5f)
-  // one lattice row; V_{m-1} of row y in `cur`, row y+1 loaded into `nxt`
-  // (the caller alternates the two register sets, so the loads issued here
-  // are first used a full row later); false when the CTA gives up
-  auto row = [&](int q, ulonglong2 (&cur)[2][2], ulonglong2 (&nxt)[2][2]) -> bool {
-    const int y = y0 + q;
-    if (__any_sync(0xffffffffu, *fail_flag != 0)) return false;
-    const int rot_next = next_rot(rot);
-    if (MODE == 1 && q + 1 < nrow) load_prev(y + 1, rot_next, nxt);
-    bool ok = true;
-    if (q == 0) ok = step_wait<HOOK>(vbar(0), 0) && step_wait<HOOK>(vbar(1), 0);
-    ok = ok && step_wait<HOOK>(vbar(q + 2), vpar(q + 2)) && step_wait<HOOK>(cbar(q), cpar(q));
-    if (threadIdx.x == 0 && ok) {
-      // window row y+3 into the slot of y-2 and coefficients of y+2 into the
-      // slot of y-1, once every warp has finished row y-1 (row 0: fresh slots)
-      if (q >= 1) ok = step_wait<HOOK>(dbar(q - 1), dpar(q - 1));
-      if (ok) {
-        if (q + 4 <= nrow + 1) issue_v(q + 4);
-        if (q + 2 < nrow) issue_c(q + 2);
-      }
-    }
-    if (!__all_sync(0xffffffffu, ok)) {
-      *fail_flag = 1;
-      return false;
-    }
-    const float4* wm = win + (q % 5) * rowsz + v;
-    const float4* w0 = win + ((q + 1) % 5) * rowsz + v;
-    const float4* wp = win + ((q + 2) % 5) * rowsz + v;
-    const float2* cf_row = coef + (q % 3) * crow;
-    const int x1 = site1(rot);
-
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      if (!(it == 0 ? own0 : x1 >= 0)) continue;
-      const int x = it == 0 ? xs : x1;
-      ulonglong2 o0, o1;
-      stencil_site<NV>(wm, w0, wp, cf_row, x, nx, o0, o1);
-      if (MODE == 1) {
-        o0.x = f2sub(o0.x, cur[it][0].x);
-        o0.y = f2sub(o0.y, cur[it][0].y);
-        o1.x = f2sub(o1.x, cur[it][1].x);
-        o1.y = f2sub(o1.y, cur[it][1].y);
-      } else {
-        o0.x = f2mul(o0.x, half2);
-        o0.y = f2mul(o0.y, half2);
-        o1.x = f2mul(o1.x, half2);
-        o1.y = f2mul(o1.y, half2);
-      }
-      float4* g = Vout + (2 * ((int64_t)y * nx + x)) * ldq + q0 + v;
-      *reinterpret_cast<ulonglong2*>(g) = o0;
-      *reinterpret_cast<ulonglong2*>(g + ldq) = o1;
-    }
-
-    if (MODE == 1 && acc != nullptr && y >= yj_lo && y <= yj_hi)
-      moment_sums<CB>(wm - v, w0 - v, wp - v, nx, y, D, cmap, cb0, m, am[m], ao[m], acc);
-    __syncwarp();
-    if (lane == 0) mbar_arrive(dbar(q));
-    rot = rot_next;
-    return true;
-  };
-  for (int q = 0; q < nrow; q += 2) {
-    if (!row(q, pc, pn)) break;
-    if (q + 1 < nrow && !row(q + 1, pn, pc)) break;
-  }
-  __syncthreads();
-  if (*fail_flag) {
-    // every copy the CTA issued may still be in flight: wait (bounded) for
-    // the last fill of every slot before the shared memory is released
-    if (threadIdx.x == 0) {
-      atomicOr(&g_step_fault, 1u);
-      for (int w = max(0, w_hi - 4); w <= w_hi; ++w) step_wait<HOOK>(vbar(w), vpar(w), 2);
-      for (int c = max(0, c_hi - 2); c <= c_hi; ++c) step_wait<HOOK>(cbar(c), cpar(c), 2);
-    }
-    __syncthreads();
-    poison();
-  }
-}
-
-template <int CB, int MODE, bool HOOK = false>
-__global__ void __launch_bounds__(512, 1)
-    cheb_step_f32_tma_kernel(const __grid_constant__ CUtensorMap tm, int nx, int ny, int64_t D, int64_t ldv,
-                             int ylen, int brows, const float2* __restrict__ table, const float4* Vprev, float4* Vout,
-                             ColMap cmap, double2* __restrict__ acc, const double* __restrict__ am,
-                             const double* __restrict__ ao, int m) {
-  f32_step_body_tma<CB, MODE, HOOK>(&tm, nx, ny, D, ldv, ylen, brows, table, Vprev, Vout, cmap, acc, am, ao, m);
 }
 
 #include "cheb_march.cuh"
@@ -1134,6 +878,10 @@ __global__ void cheb_init_acc_kernel(int64_t D, int64_t ldv, int nx, ColMap cm, 
     double2 a = make_double2(0.0, 0.0);
     if (s == 0) a.x = am[0];
     if (s == kSlots - 1) a.x = ao[0];
+    if (cm.raw) {  // times xi_J, which the gather takes out again
+      const double2 x = cm.xi[J];
+      a = make_double2(a.x * x.x, -a.x * x.y);
+    }
     acc[J * kSlots + s] = a;
     if (s == 0 && cm.rec) cm.rec[(J & 1) * (D >> 1) + (J >> 1)] = 1.0;  // T_0 = 1
   }
@@ -1143,6 +891,45 @@ __global__ void probe_phase_kernel(int64_t D, uint32_t seed, double2* __restrict
   for (int64_t K = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; K < D; K += (int64_t)gridDim.x * blockDim.x) {
     const double2 x = probe_xi(seed, K);
     xi_conj[K] = make_double2(x.x, -x.y);
+  }
+}
+
+// Moment sums of a probing slab, V_m = Va and (if given) V_{m+1} = Vb, one thread
+// per source and slot.  Every row is a source, and a march CTA meets its share of them in
+// bursts (all the sites of every p-th row): in the march's sums warp they held its
+// rings up for 6 to 18 us a step.  Here two moments go into one update of the sums, kept
+// without the phase conj(xi_J), which the gather multiplies in: four FP64 operations a
+// moment and slot pair less than weighting every term (the FP64 pipe is 1/64 of FP32's).
+__global__ void probe_sums_kernel(int nx, int ny, int D, int64_t ldv, const float4* __restrict__ Va,
+                                  const float4* __restrict__ Vb, ColMap cm, double2* __restrict__ acc,
+                                  const double* __restrict__ am, const double* __restrict__ ao, int m) {
+  const int p = cm.probe_p;
+  const int64_t ldq = ldv / 2;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < D * kSlots; t += gridDim.x * blockDim.x) {
+    const int J = t / kSlots, s = t - J * kSlots;
+    const int i = J >> 1, y = i / nx, x = i - y * nx;
+    const int c = (J & 1) + 2 * (x % p + p * (y % p)) - (int)cm.s0;
+    if (c < 0 || c >= ldv) continue;
+    int xs = x + kSlotDx[s], ys = y + kSlotDy[s];
+    xs = xs < 0 ? xs + nx : xs >= nx ? xs - nx : xs;
+    ys = ys < 0 ? ys + ny : ys >= ny ? ys - ny : ys;
+    const int64_t K = 2 * (ys * nx + xs) + ((J & 1) ^ kSlotFlip[s]);
+    const int64_t at = 4 * (K * ldq + (c >> 1)) + (c & 1);
+    double2 a = acc[t];
+    const double* const cf = s == kSlots - 1 ? ao : am;
+    const float ar = reinterpret_cast<const float*>(Va)[at], ai = reinterpret_cast<const float*>(Va)[at + 2];
+    float br = 0.f, bi = 0.f;
+    if (Vb) {
+      br = reinterpret_cast<const float*>(Vb)[at];
+      bi = reinterpret_cast<const float*>(Vb)[at + 2];
+    }
+    acc_add_unit(&a, cf[m], (double)ar, (double)ai);
+    if (Vb) acc_add_unit(&a, cf[m + 1], (double)br, (double)bi);
+    acc[t] = a;
+    if (s == 0 && cm.rec) {
+      record_diag(cm, D, m, J, cm.xi[J], (double)ar, (double)ai);
+      if (Vb) record_diag(cm, D, m + 1, J, cm.xi[J], (double)br, (double)bi);
+    }
   }
 }
 
@@ -1188,7 +975,15 @@ __global__ void cheb_gather_kernel(int nx, int ny, int64_t D, int64_t ldv, int64
       re = val.x;
       im = val.y;
     }
-    acc_add(acc + J * kSlots + s, s == kSlots - 1 ? ao[m] : am[m], wgt, re, im);
+    double2* const e = acc + J * kSlots + s;
+    const double coef = s == kSlots - 1 ? ao[m] : am[m];
+    if (cm.raw) {  // sums kept without the phase: conj(xi_J) (sum + the last term)
+      double2 t = *e;
+      acc_add_unit(&t, coef, re, im);
+      *e = make_double2(wgt.x * t.x - wgt.y * t.y, wgt.x * t.y + wgt.y * t.x);
+    } else {
+      acc_add(e, coef, wgt, re, im);
+    }
     if (s == 0 && cm.rec) record_diag(cm, D, m, J, wgt, re, im);
   }
 }
@@ -1441,9 +1236,7 @@ __global__ void __cluster_dims__(kPClu, 1, 1) __launch_bounds__(512, 1)
 }
 
 constexpr size_t kSmemLimit = 227 * 1024;
-// mbarriers of the TMA step (5 window + 3 coefficient slots + 3 row-done) and its fault flag
-constexpr size_t kTmaBarBytes = 16 * sizeof(uint64_t);
-// host side: launch the test-hook instantiation of the TMA step (set by
+// host side: launch the test-hook instantiation of the march kernel (set by
 // set_step_failure_test; launches enqueued or captured after it)
 bool g_step_hook_armed = false;
 constexpr int kSMs = 152;
@@ -1464,14 +1257,7 @@ cudaError_t set_smem_f32(int nx) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(cheb_step_f32_kernel<CB, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)kSmemLimit);
-  if (e != cudaSuccess || CB < 8) return e;
-  constexpr int CT = CB >= 8 ? CB : 8;
-  for (auto fn : {cheb_step_f32_tma_kernel<CT, 0, false>, cheb_step_f32_tma_kernel<CT, 1, false>,
-                  cheb_step_f32_tma_kernel<CT, 0, true>, cheb_step_f32_tma_kernel<CT, 1, true>}) {
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return e;
 }
 
 // cuTensorMapEncodeTiled, resolved once through the runtime's driver entry point
@@ -1519,20 +1305,6 @@ template <int CB>
 cudaError_t launch_f32(const ChebPlan& p, const void* table, const void* Vcur, const void* Vprev, void* Vout,
                        int64_t s0, double2* acc, const double* am, const double* ao, int m, int mode, cudaStream_t s) {
   const dim3 grid((p.ny + p.ylen - 1) / p.ylen, (unsigned)(p.ldv / CB));
-  if (CB >= 8 && p.tma_rows > 0) {
-    constexpr int CT = CB >= 8 ? CB : 8;
-    CUtensorMap tm;
-    const cudaError_t e = encode_slab_map(&tm, Vcur, p.D, p.ldv, CB, p.tma_rows);
-    if (e != cudaSuccess) return e;
-    const size_t sm = p.smem + kTmaBarBytes;
-    // the failure-path test instantiation only while a test hook is armed
-    auto fn = g_step_hook_armed ? (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, true> : cheb_step_f32_tma_kernel<CT, 1, true>)
-                                : (mode == 0 ? cheb_step_f32_tma_kernel<CT, 0, false>
-                                             : cheb_step_f32_tma_kernel<CT, 1, false>);
-    fn<<<grid, p.nthreads, sm, s>>>(tm, p.nx, p.ny, p.D, p.ldv, p.ylen, p.tma_rows, (const float2*)table,
-                                    (const float4*)Vprev, (float4*)Vout, colmap(p, s0), acc, am, ao, m);
-    return cudaGetLastError();
-  }
   if (mode == 0)
     cheb_step_f32_kernel<CB, 0><<<grid, p.nthreads, p.smem, s>>>(p.nx, p.ny, p.D, p.ldv, p.ylen, (const float2*)table,
                                                                  (const float4*)Vcur, (const float4*)Vprev, (float4*)Vout,
@@ -1595,12 +1367,28 @@ cudaError_t set_smem_march() {
   return cudaSuccess;
 }
 template <int NV, int NS>
-void march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, const MarchMaps& pr, const MarchArgs& a,
+cudaError_t march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, const MarchMaps& pr, const MarchArgs& a,
                   const ColMap& cm, bool first, cudaStream_t s) {
   // the failure-path test instantiation only while a test hook is armed
   auto fn = g_step_hook_armed ? (first ? cheb_march_kernel<NV, NS, true, true> : cheb_march_kernel<NV, NS, false, true>)
                               : (first ? cheb_march_kernel<NV, NS, true, false> : cheb_march_kernel<NV, NS, false, false>);
-  fn<<<grid, mp.warps * 32, mp.smem, s>>>(v, pr, a, cm);
+  // Outside graphs the launches are programmatic: a CTA's start runs while the launch
+  // before finishes, and the kernel waits for that before it touches anything (37x29,
+  // 776 steps: 16.1 -> 14.3 ms; as nodes of a graph, 48x24, the same cost 3%).
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &cap);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)(mp.warps * 32));
+  cfg.dynamicSmemBytes = mp.smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, v, pr, a, cm);
 }
 }  // namespace
 
@@ -1727,10 +1515,9 @@ cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* tab
   memcpy(&pr, prev.p, sizeof(pr));
   const dim3 grid((unsigned)(((p.ny + mp.ylen - 1) / mp.ylen) * mp.ntile), (unsigned)(p.ldv / (2 * kMarchPairs)));
   const ColMap cm = colmap(p, s0);
-  if (mp.ns == 1) march_launch<kMarchPairs, 1>(mp, grid, v, pr, a, cm, first, s);
-  else if (mp.ns == 2) march_launch<kMarchPairs, 2>(mp, grid, v, pr, a, cm, first, s);
-  else march_launch<kMarchPairs, 3>(mp, grid, v, pr, a, cm, first, s);
-  return cudaGetLastError();
+  if (mp.ns == 1) return march_launch<kMarchPairs, 1>(mp, grid, v, pr, a, cm, first, s);
+  if (mp.ns == 2) return march_launch<kMarchPairs, 2>(mp, grid, v, pr, a, cm, first, s);
+  return march_launch<kMarchPairs, 3>(mp, grid, v, pr, a, cm, first, s);
 }
 
 // Wave model of a launch: ctas x nb CTAs (nb bands of ceil(ny/nb) rows) run
@@ -1765,13 +1552,13 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
   p.cb = 0;
   p.ldv = 0;
   p.smem = 0;
-  p.tma_rows = 0;
   p.ylen = ny;
   p.js = 0;
   p.probe_p = 0;
   p.probe_seed = 0;
   p.xi = nullptr;
   p.rec = nullptr;
+  p.raw = 0;
   // widest column chunk that fits shared memory (FP32: 16 columns, FP64: 8);
   // FP32 also needs every thread to own at most two sites of a lattice row
   const int cands32[4] = {16, 8, 4, 2};
@@ -1795,7 +1582,7 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
     }
   }
   if (precision == KPM_FP32 && steps > 0 && p.cb > 0) {
-    // unit vectors: the march kernel, for every lattice whose row the one-step kernels take
+    // the march kernel, for every lattice whose row the one-step kernels take
     p.cb = 2 * kMarchPairs;
     p.ldv = (width + p.cb - 1) / p.cb * p.cb;
     p.m1 = plan_march(nx, ny, p.ldv, 1, band_rows);
@@ -1805,17 +1592,6 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
     p.nthreads = 32 * p.mk.warps;
     p.smem = p.mk.smem;
     return p;
-  }
-  if (precision == KPM_FP32 && p.cb >= 8 && p.smem + kTmaBarBytes <= kSmemLimit) {
-    // TMA staging: the 2 Nx Nambu rows of a window row in nb equal boxes of
-    // at most 256 rows, each landing on a 128-byte boundary of shared memory
-    const int rows = 2 * nx;
-    for (int nb = (rows + 255) / 256; nb <= rows; ++nb) {
-      if (rows % nb) continue;
-      const int br = rows / nb;
-      if ((br * p.cb * 8) % 128 == 0) p.tma_rows = br;
-      break;
-    }
   }
   if (p.cb == 0) return p;
   p.ldv = (width + p.cb - 1) / p.cb * p.cb;
@@ -1848,8 +1624,9 @@ size_t table_bytes_per_site(int precision) { return (size_t)kCoef * (precision =
 
 cudaError_t cheb_prepare(const ChebPlan& p, int precision) {
   if (p.mk.ns) {
-    const cudaError_t e = march_prepare(p.mk);
-    return e != cudaSuccess ? e : march_prepare(p.m1);
+    cudaError_t e = march_prepare(p.mk);
+    if (e == cudaSuccess) e = march_prepare(p.m1);
+    return e;
   }
   if (precision == KPM_FP32) {
     switch (p.cb) {
@@ -1950,6 +1727,15 @@ cudaError_t set_step_failure_test(int drop_copies, uint64_t wait_limit_ns) {
 cudaError_t launch_probe_phases(const ChebPlan& p, double2* xi_conj, cudaStream_t s) {
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((p.D + 255) / 256, 4 * kSMs));
   probe_phase_kernel<<<grid, 256, 0, s>>>(p.D, p.probe_seed, xi_conj);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_probe_sums(const ChebPlan& p, const void* Va, const void* Vb, int64_t s0, double2* acc,
+                              const double* am, const double* ao, int m, cudaStream_t s) {
+  const int64_t n = p.D * kSlots;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 8 * kSMs));
+  probe_sums_kernel<<<grid, 256, 0, s>>>(p.nx, p.ny, (int)p.D, p.ldv, (const float4*)Va, (const float4*)Vb,
+                                         colmap(p, s0), acc, am, ao, m);
   return cudaGetLastError();
 }
 

@@ -1,5 +1,4 @@
-// FP32 recursion steps on unit vectors, NS steps per launch (included by
-// cheb_kernels.cu).
+// FP32 recursion steps, NS steps per launch (included by cheb_kernels.cu).
 //
 // One CTA runs NS consecutive Chebyshev steps of a tile: CB = 2 NV columns, tx
 // sites of the lattice rows (the whole row where it fits: `full`) and the
@@ -31,7 +30,7 @@
 // number of the recursion has the same bits whatever NS, tile and band.
 //
 // Measured against the one-step kernel with block-shared windows, us per step:
-// 37x29 40.0 -> 20.8, 48x24 31.8 -> 16.7 (one step, slabs in L2), 64x64 343 ->
+// 37x29 40.0 -> 20.8 (18.3 where launches overlap), 48x24 31.8 -> 16.7 (one step, slabs in L2), 64x64 343 ->
 // 266 (one step, 90% of the copy rate), 100x100 1655 -> 1248 (two steps; one
 // step: 1457 = 97% of the copy rate), its eighth (2500 columns) 237 -> 180.
 //
@@ -43,7 +42,7 @@
 // or, s > 0, row i + 2 of stage s - 1's input; the sums read input rows i .. i + 2.
 // A set is issued once the last stage has finished row i - lag, so stage s row
 // i - lag + 2 (NS - 1 - s); the ring sizes follow (plan_march) and a test replays
-// them.  Every wait is bounded (see step_wait): a CTA whose waits run out writes
+// them.  Every wait is bounded: a CTA whose waits run out writes
 // NaN over the rows and columns it owns.
 
 constexpr int kMarchPairs = 8;      // column pairs per CTA
@@ -212,7 +211,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     return __all_sync(0xffffffffu, march_wait_slow(bar, parity(i), limit(), fail)) != 0;
   };
 
+  // launched programmatically, a CTA starts while the launch before finishes: it touches
+  // no slab, sum or entry before this
+  auto grid_wait = [&]() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); };
   auto poison = [&]() {  // NaN over the tile's outputs
+    grid_wait();
     const float nan = __int_as_float(0x7fc00000);
     const float4 nan4 = make_float4(nan, nan, nan, nan);
     for (int t = threadIdx.x; t < nrow * 2 * w * NV; t += blockDim.x) {
@@ -222,6 +225,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
       a.outb[g] = nan4;
     }
   };
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   // after a fault anywhere, later CTAs and launches only mark their outputs
   if (*reinterpret_cast<volatile unsigned int*>(&g_step_fault) != 0u) {
     poison();
@@ -241,6 +245,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     poison();
     return;
   }
+
+  grid_wait();
 
   if (warp == first_warp[NS]) {
     // producer: the sets, as soon as the ring rows they overwrite are free.  The whole

@@ -254,8 +254,8 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
     if (pp->ranged && (o->flags & KPM_FLAG_PH_HALF))
       return fail(ctx, KPM_EINVAL, "KPM_FLAG_PH_HALF and a site range do not combine");
   }
-  const bool march = o->precision == KPM_FP32 && pp_ == 0;  // FP32 unit vectors
-  const bool deeper = march && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
+  const bool march = o->precision == KPM_FP32;
+  const bool deeper = march && pp_ == 0 && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
   const int js = (o->flags & KPM_FLAG_PH_HALF) ? 1 : 0;
   // start vectors of the pass: unit columns (those of the site range), or R = 2 p^2 probing vectors
   pp->c0 = pp->ranged ? 2 * (int64_t)pp->sb : 0;
@@ -269,7 +269,7 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
     return balanced_width(ncols, std::min<int64_t>(ncols, std::max<int64_t>(fit, 1)));
   };
   int64_t width = width_of(2);
-  int steps = march ? (single ? 1 : march_steps(m->nx, m->ny, width)) : 0;
+  int steps = march ? (single || pp_ > 0 ? 1 : march_steps(m->nx, m->ny, width)) : 0;
   if (steps > 1 && (o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
   if (deeper) ++steps;
   if (steps > 1) width = width_of(4);
@@ -278,6 +278,7 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
   pp->cheb.js = js;
   pp->cheb.probe_p = pp_;
   pp->cheb.probe_seed = (uint32_t)o->probe_seed;
+  pp->cheb.raw = march && pp_ > 0 && o->M >= 2;
   if (pp->cheb.cb == 0) return fail(ctx, KPM_EINVAL, "lattice row too wide for the shared-memory window");
   // slabs advance by the padded width: every unit column belongs to exactly one slab
   pp->width = pp->cheb.ldv;
@@ -402,14 +403,19 @@ int enqueue_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, const Pass
       } else {
         // one step, in place over V_{mm-1} (the first into the second slab)
         const int io = first ? 1 : ix;
-        KPM_CU(launch_march(p, p.m1, table1, m1[iy], m1[ix], nullptr, ctx->slab[io], s0, ctx->acc, ctx->am,
-                            ctx->ao, mm, first, s));
+        KPM_CU(launch_march(p, p.m1, table1, m1[iy], m1[ix], nullptr, ctx->slab[io], s0, p.raw ? nullptr : ctx->acc,
+                            ctx->am, ctx->ao, mm, first, s));
         nb += (first ? 2 : 3) * vec;
         ix = iy;
         iy = io;
         mm += 1;
       }
       nr += 1;
+      if (p.raw && mm % 2 == 0) {  // probing: V_{mm-1} and V_mm (the gather takes V_{M-1})
+        KPM_CU(launch_probe_sums(p, ctx->slab[ix], mm < M - 1 ? ctx->slab[iy] : nullptr, s0, ctx->acc, ctx->am, ctx->ao,
+                                 mm - 1, s));
+        nl += 1;
+      }
     }
     if (events && s0 + pp.width >= pp.c1) KPM_CU(cudaEventRecordWithFlags(ctx->ev[1], s, cudaEventRecordExternal));
     if (M >= 2) {

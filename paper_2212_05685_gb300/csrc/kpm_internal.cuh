@@ -31,7 +31,7 @@ struct alignas(64) SlabMaps {
 
 // Launch geometry of the recursion kernel (shared with the host planner).
 struct ChebPlan {
-  MarchPlan mk;    // FP32 unit vectors: the pass's launches of several steps (or one)
+  MarchPlan mk;    // FP32: the pass's launches of several steps (or one)
   MarchPlan m1;    // and the single step
   int nx, ny;
   int64_t D;       // 2 N
@@ -40,7 +40,6 @@ struct ChebPlan {
   int ylen;        // lattice rows marched per CTA
   int nthreads;
   size_t smem;     // dynamic shared memory per CTA
-  int tma_rows;    // FP32 probing step: Nambu rows per TMA box of a window row (0: cp.async staging)
   // slab column c holds unit vector J = (s0 + c) << js (js = 1: particle-hole
   // half pass over the columns (j, up) only; the pass covers D >> js columns)
   int js;
@@ -50,6 +49,7 @@ struct ChebPlan {
   uint32_t probe_seed;
   const double2* xi;  // device table conj(xi_J) of the pass (probing only)
   double* rec;        // diagonal moments [T_m(h~)]_JJ, rec[m D + (J & 1) N + (J >> 1)] (or null)
+  int raw;            // probing: moment sums kept without the phase until the gather
 };
 
 // What slab column c of a launch holds (built from the plan and the slab offset).
@@ -60,8 +60,9 @@ struct ColMap {
   uint32_t seed;
   const double2* xi;  // conj(xi_J), J < D (probing)
   double* rec;        // diagonal-moment record (or null)
+  int raw;            // probing: sums without the phase
 };
-inline ColMap colmap(const ChebPlan& p, int64_t s0) { return ColMap{s0, p.js, p.probe_p, p.probe_seed, p.xi, p.rec}; }
+inline ColMap colmap(const ChebPlan& p, int64_t s0) { return ColMap{s0, p.js, p.probe_p, p.probe_seed, p.xi, p.rec, p.raw}; }
 // unit start vectors (D >> js) or probing vectors (2 p^2) of a pass
 inline int64_t pass_columns(const ChebPlan& p) {
   return p.probe_p > 0 ? 2 * (int64_t)p.probe_p * p.probe_p : (p.D >> p.js);
@@ -124,8 +125,8 @@ cudaError_t launch_update(int N, double* params, double* obs, double* mu_eff, co
 int reduce_scratch_doubles(int64_t n);
 
 // ---------------------------------------------------------------- cheb_kernels.cu
-// steps: FP32 recursion steps per launch of unit-vector slabs (the march kernel,
-// chunks of 16 columns); 0: the one-step kernels of probing slabs, FP64 and double-float
+// steps: FP32 recursion steps per launch of the march kernel (chunks of 16 columns);
+// 0: the one-step kernels (FP64, double-float, narrower FP32 chunks)
 ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0, int steps = 0);
 // FP32 steps per launch at which unit-vector slabs of `width` columns run fastest
 int march_steps(int nx, int ny, int64_t width);
@@ -147,11 +148,11 @@ cudaError_t launch_cheb_init(const ChebPlan& p, int precision, void* V0, int64_t
 cudaError_t launch_cheb_step(const ChebPlan& p, int precision, const void* table, const void* Vcur,
                              void* Vout, int64_t s0, double2* acc, const double* am,
                              const double* ao, int m, int mode, cudaStream_t s, const void* Vprev = nullptr);
-// device fault word of the TMA-staged FP32 steps (bit 0: a bounded wait
+// device fault word of the FP32 march kernel (bit 0: a bounded wait
 // expired; bit 1: shared memory misaligned for TMA); sticky for the process
 cudaError_t read_step_fault(unsigned int* out);
 cudaError_t clear_step_fault();
-// failure-path test hook: the next drop_copies CTAs of the TMA step skip one
+// failure-path test hook: the next drop_copies CTAs of the march kernel skip one
 // window copy; bounded-wait limit of later launches (0: the default 2 s)
 cudaError_t set_step_failure_test(int drop_copies, uint64_t wait_limit_ns);
 // FP32 march: tensor maps of a slab, and one launch of mp.ns steps from V_m = Vcur
@@ -166,6 +167,9 @@ cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* tab
 size_t march_table_bytes(const MarchPlan& mp, int ny);
 // table conj(xi_J) of the probing phases, J < D
 cudaError_t launch_probe_phases(const ChebPlan& p, double2* xi_conj, cudaStream_t s);
+// FP32 probing slab: moment sums of V_m = Va and, if Vb, of V_{m+1} = Vb (p.raw)
+cudaError_t launch_probe_sums(const ChebPlan& p, const void* Va, const void* Vb, int64_t s0, double2* acc,
+                              const double* am, const double* ao, int m, cudaStream_t s);
 // acc += a_m V[local rows] for the slab's columns (no recursion)
 cudaError_t launch_cheb_gather(const ChebPlan& p, int precision, const void* V, int64_t s0,
                                double2* acc, const double* am, const double* ao, int m,

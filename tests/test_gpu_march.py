@@ -99,3 +99,14 @@ def test_default_steps_shrink_to_the_budget(K):
         assert np.array_equal(got[:-1], ref[:-1])
     finally:
         kpm.kpm_destroy(ctx)
+
+
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 12])
+@pytest.mark.parametrize("nx,ny,p,bw", [(2, 2, 2, 0), (12, 8, 4, 0), (12, 12, 3, 8), (60, 3, 3, 16)])
+def test_probing_sums_of_every_order(K, nx, ny, p, bw, M):
+    """FP32 probing keeps its moment sums two moments a launch, without the phase until the last
+    moment: every remainder of the order, one and several slabs, against the FP64 pass of the same
+    vectors (one-step kernels), within the FP32 tolerance of the other tests."""
+    cell = _cell(K, nx, ny)
+    kw = dict(block_width=bw, probe_p=p, probe_seed=3)
+    assert np.max(np.abs(_pass(K, cell, M, 1, **kw)[:-1] - _pass(K, cell, M, 0, **kw)[:-1])) < 2e-5
