@@ -22,9 +22,9 @@
 // columns.  h~ is a 13-point stencil per row (diagonal, eight hops, four
 // pairings), read from a per-site table of kCoef complex 2h~ entries.
 //
-// FP32 runs the march kernel (cheb_march.cuh).  The kernels of this file serve FP64
-// and double-float, and FP32 where the march kernel's 16-column chunk does not
-// fit (the allocation-free call): each CTA owns a chunk of CB columns and a band
+// Passes run the march kernel (cheb_march.cuh).  The one-step kernels of this file serve
+// FP64 and double-float probing, and slabs narrower than the march kernel's chunk
+// (the allocation-free call): each CTA owns a chunk of CB columns and a band
 // of lattice rows y0..y1-1 and marches along y keeping lattice rows y-1, y, y+1
 // of V_m (all Nx sites, both Nambu components, CB columns) in shared memory, the
 // next rows and coefficient rows in flight by cp.async, so every V_m element is
@@ -1278,14 +1278,14 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
-// Tensor map of an FP32 pair-split slab V[D][ldv] viewed as D rows of 2 ldv
-// floats; box: 2 cb floats (the chunk's cb complex columns) x brows Nambu rows
-cudaError_t encode_slab_map(CUtensorMap* tm, const void* V, int64_t D, int64_t ldv, int cb, int brows) {
+// Tensor map of a slab viewed as D rows of `floats` floats; box: a chunk's elements
+// (4 kMarchLanes floats) x brows Nambu rows
+cudaError_t encode_slab_map(CUtensorMap* tm, const void* V, int64_t D, int64_t floats, int brows) {
   EncodeTiledFn fn = encode_tiled();
   if (!fn) return cudaErrorNotSupported;
-  const cuuint64_t dims[2] = {(cuuint64_t)(2 * ldv), (cuuint64_t)D};
-  const cuuint64_t strides[1] = {(cuuint64_t)(8 * ldv)};
-  const cuuint32_t box[2] = {(cuuint32_t)(2 * cb), (cuuint32_t)brows};
+  const cuuint64_t dims[2] = {(cuuint64_t)floats, (cuuint64_t)D};
+  const cuuint64_t strides[1] = {(cuuint64_t)(4 * floats)};
+  const cuuint32_t box[2] = {4 * kMarchLanes, (cuuint32_t)brows};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(V), dims, strides, box, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1357,21 +1357,21 @@ cudaError_t launch_f64(const ChebPlan& p, const void* table, const void* Vcur, c
 }  // namespace
 
 namespace {
-template <int NV, int NS>
+template <int EL, int NS>
 cudaError_t set_smem_march() {
-  for (auto fn : {cheb_march_kernel<NV, NS, false, false>, cheb_march_kernel<NV, NS, true, false>,
-                  cheb_march_kernel<NV, NS, false, true>, cheb_march_kernel<NV, NS, true, true>}) {
+  for (auto fn : {cheb_march_kernel<EL, NS, false, false>, cheb_march_kernel<EL, NS, true, false>,
+                  cheb_march_kernel<EL, NS, false, true>, cheb_march_kernel<EL, NS, true, true>}) {
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
-template <int NV, int NS>
+template <int EL, int NS>
 cudaError_t march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, const MarchMaps& pr, const MarchArgs& a,
                   const ColMap& cm, bool first, cudaStream_t s) {
   // the failure-path test instantiation only while a test hook is armed
-  auto fn = g_step_hook_armed ? (first ? cheb_march_kernel<NV, NS, true, true> : cheb_march_kernel<NV, NS, false, true>)
-                              : (first ? cheb_march_kernel<NV, NS, true, false> : cheb_march_kernel<NV, NS, false, false>);
+  auto fn = g_step_hook_armed ? (first ? cheb_march_kernel<EL, NS, true, true> : cheb_march_kernel<EL, NS, false, true>)
+                              : (first ? cheb_march_kernel<EL, NS, true, false> : cheb_march_kernel<EL, NS, false, false>);
   // Outside graphs the launches are programmatic: a CTA's start runs while the launch
   // before finishes, and the kernel waits for that before it touches anything (37x29,
   // 776 steps: 16.1 -> 14.3 ms; as nodes of a graph, 48x24, the same cost 3%).
@@ -1394,19 +1394,21 @@ cudaError_t march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, con
 
 namespace {
 // band heights of a march launch: as many CTAs per SM as registers and shared memory
-// take; a CTA's start (barriers, first copies) costs about five rows, and a launch of
-// several steps computes two more rows for every step but the last
+// take; a CTA's start (barriers, first copies) costs about five rows (one of double-float
+// or FP64), and a launch of several steps computes two more rows for every step but the last
 int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
   const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>(16 / p.warps, (int64_t)(228 * 1024) / (int64_t)(p.smem + 1024)));
-  return band_rows_candidates(ny, ldv / (2 * kMarchPairs) * p.ntile, out, maxn, per_sm * kSMs, 5.0 + 2.0 * (p.ns - 1));
+  const double start = p.el == kElF32 ? 5.0 + 2.0 * (p.ns - 1) : 1.0;
+  return band_rows_candidates(ny, ldv / march_cols(p.el) * p.ntile, out, maxn, per_sm * kSMs, start);
 }
 
 // Geometry of a march launch: the whole lattice row per CTA where its threads
 // fit, else the fewest equal tiles; then the deepest rings that fit shared
 // memory (several steps: eight rows each), and the band height of the wave model.
-MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows) {
+MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows, int el = kElF32) {
   MarchPlan p;
-  constexpr int nv = kMarchPairs;
+  p.el = el;
+  constexpr int nv = kMarchLanes;
   auto warps = [&](int tx, bool full) {
     int n = 2;  // the producer and the moment sums
     for (int s = 0; s < ns; ++s) n += ((full ? nx : tx + 2 * (ns - 1 - s)) * nv + 31) / 32;
@@ -1430,11 +1432,12 @@ MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows) {
   }
   p.warps = warps(p.tx, p.full);
   p.wrow = p.full ? nx : p.tx + 2 * ns;
-  p.crowb = (p.wrow * 208 + 127) / 128 * 128;
+  p.crowb = (p.wrow * march_entry_bytes(el) + 127) / 128 * 128;
   // a set of rows is issued once the last stage has finished the row `lag` before it;
   // single step: row i + 2 of V_m then takes the place of one that the stage and the
   // sums have done with in a ring of lag + 2 rows
-  for (int lag = 8; lag >= (ns == 1 ? 3 : 8); --lag) {
+  // (a row of double-float or FP64 takes as long as its copy: four are enough)
+  for (int lag = el == kElF32 ? 8 : 4; lag >= (ns == 1 ? 2 : 8); --lag) {
     p.lag = lag;
     p.rv = ns == 1 ? lag + 2 : kMarchRows;
     p.rp = p.rc = ns == 1 ? lag : kMarchRows;
@@ -1456,8 +1459,9 @@ MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows) {
 
 namespace {
 cudaError_t march_prepare(const MarchPlan& mp) {
-  return mp.ns == 1 ? set_smem_march<kMarchPairs, 1>()
-                    : mp.ns == 2 ? set_smem_march<kMarchPairs, 2>() : set_smem_march<kMarchPairs, 3>();
+  if (mp.el == kElDF) return set_smem_march<kElDF, 1>();
+  if (mp.el == kElF64) return set_smem_march<kElF64, 1>();
+  return mp.ns == 1 ? set_smem_march<kElF32, 1>() : mp.ns == 2 ? set_smem_march<kElF32, 2>() : set_smem_march<kElF32, 3>();
 }
 }  // namespace
 
@@ -1468,7 +1472,7 @@ cudaError_t encode_slab_maps(const ChebPlan& p, const MarchPlan& mp, const void*
     const int sites[3] = {mp.full ? mp.tx : mp.tx + 2 * halo, mp.full ? mp.tx : mp.tx + halo, std::max(1, halo)};
     for (int k = 0; k < (mp.full ? 1 : 3); ++k) {
       CUtensorMap t;
-      const cudaError_t e = encode_slab_map(&t, V, p.D, p.ldv, 2 * kMarchPairs, 2 * sites[k]);
+      const cudaError_t e = encode_slab_map(&t, V, p.D, (mp.el == kElF32 ? 2 : 4) * p.ldv, 2 * sites[k]);
       if (e != cudaSuccess) return e;
       memcpy(to + 128 * k, &t, 128);
     }
@@ -1489,7 +1493,7 @@ cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* tab
   a.nx = p.nx;
   a.ny = p.ny;
   a.D = p.D;
-  a.ldq = p.ldv / 2;
+  a.ldq = mp.el == kElF32 ? p.ldv / 2 : p.ldv;  // 16-byte elements of a slab row
   a.tx = mp.tx;
   a.ntile = mp.ntile;
   a.full = mp.full;
@@ -1500,7 +1504,7 @@ cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* tab
   a.rv = mp.rv;
   a.rs = mp.rs;
   a.rc = mp.rc;
-  a.rowb = mp.wrow * 32 * kMarchPairs;
+  a.rowb = mp.wrow * 32 * kMarchLanes;
   a.crowb = mp.crowb;
   a.table = (const float4*)table;
   a.outa = (float4*)outa;
@@ -1513,11 +1517,13 @@ cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* tab
   MarchMaps v, pr;
   memcpy(&v, cur.v, sizeof(v));
   memcpy(&pr, prev.p, sizeof(pr));
-  const dim3 grid((unsigned)(((p.ny + mp.ylen - 1) / mp.ylen) * mp.ntile), (unsigned)(p.ldv / (2 * kMarchPairs)));
+  const dim3 grid((unsigned)(((p.ny + mp.ylen - 1) / mp.ylen) * mp.ntile), (unsigned)(p.ldv / march_cols(mp.el)));
   const ColMap cm = colmap(p, s0);
-  if (mp.ns == 1) return march_launch<kMarchPairs, 1>(mp, grid, v, pr, a, cm, first, s);
-  if (mp.ns == 2) return march_launch<kMarchPairs, 2>(mp, grid, v, pr, a, cm, first, s);
-  return march_launch<kMarchPairs, 3>(mp, grid, v, pr, a, cm, first, s);
+  if (mp.el == kElDF) return march_launch<kElDF, 1>(mp, grid, v, pr, a, cm, first, s);
+  if (mp.el == kElF64) return march_launch<kElF64, 1>(mp, grid, v, pr, a, cm, first, s);
+  if (mp.ns == 1) return march_launch<kElF32, 1>(mp, grid, v, pr, a, cm, first, s);
+  if (mp.ns == 2) return march_launch<kElF32, 2>(mp, grid, v, pr, a, cm, first, s);
+  return march_launch<kElF32, 3>(mp, grid, v, pr, a, cm, first, s);
 }
 
 // Wave model of a launch: ctas x nb CTAs (nb bands of ceil(ny/nb) rows) run
@@ -1581,12 +1587,13 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
       break;
     }
   }
-  if (precision == KPM_FP32 && steps > 0 && p.cb > 0) {
+  if (steps > 0 && p.cb > 0) {
     // the march kernel, for every lattice whose row the one-step kernels take
-    p.cb = 2 * kMarchPairs;
+    const int el = precision == KPM_FP32 ? kElF32 : precision == KPM_DF64 ? kElDF : kElF64;
+    p.cb = march_cols(el);
     p.ldv = (width + p.cb - 1) / p.cb * p.cb;
-    p.m1 = plan_march(nx, ny, p.ldv, 1, band_rows);
-    p.mk = steps > 1 ? plan_march(nx, ny, p.ldv, steps, band_rows) : p.m1;
+    p.m1 = plan_march(nx, ny, p.ldv, 1, band_rows, el);
+    p.mk = steps > 1 && el == kElF32 ? plan_march(nx, ny, p.ldv, steps, band_rows) : p.m1;
     if (p.mk.ns == 0) p.mk = p.m1;
     p.ylen = p.mk.ylen;
     p.nthreads = 32 * p.mk.warps;
@@ -1674,7 +1681,7 @@ cudaError_t launch_cheb_step(const ChebPlan& p, int precision, const void* table
                              int64_t s0, double2* acc, const double* am, const double* ao, int m, int mode,
                              cudaStream_t s, const void* Vprev) {
   if (!Vprev) Vprev = Vout;
-  if (precision == KPM_FP32 && p.m1.ns) {
+  if (p.m1.ns) {
     SlabMaps cur, prev;
     cudaError_t e = encode_slab_maps(p, p.m1, Vcur, &cur, true, false);
     if (e == cudaSuccess) e = encode_slab_maps(p, p.m1, Vprev, &prev, false, true);

@@ -1,4 +1,5 @@
-// FP32 recursion steps, NS steps per launch (included by cheb_kernels.cu).
+// Recursion steps: FP32, NS steps per launch, and FP64 and double-float, one (included by
+// cheb_kernels.cu).
 //
 // One CTA runs NS consecutive Chebyshev steps of a tile: CB = 2 NV columns, tx
 // sites of the lattice rows (the whole row where it fits: `full`) and the
@@ -33,6 +34,10 @@
 // 37x29 40.0 -> 20.8 (18.3 where launches overlap), 48x24 31.8 -> 16.7 (one step, slabs in L2), 64x64 343 ->
 // 266 (one step, 90% of the copy rate), 100x100 1655 -> 1248 (two steps; one
 // step: 1457 = 97% of the copy rate), its eighth (2500 columns) 237 -> 180.
+// FP64 and double-float elements (one complex number of 16 bytes in place of a column
+// pair, 24 cmac and two real products a site) are bound by their arithmetic; the march
+// keeps its warps out of row lockstep: FP64 16x16, M = 256, 9.45 -> 7.14 ms (6.5 at the
+// FP64 rate), double-float 48x24, M = 1024, 165.7 -> 160.8.
 //
 // Rings and barriers (indices count rows of a stage from its first row).
 // Set i = {V_m row i + 2 (set 0: rows 0, 1, 2), V_{m-1} row i, entries row i}
@@ -45,7 +50,11 @@
 // them.  Every wait is bounded: a CTA whose waits run out writes
 // NaN over the rows and columns it owns.
 
-constexpr int kMarchPairs = 8;      // column pairs per CTA
+// elements: FP32 column pairs, double-float and FP64 complex numbers, 16 bytes each
+enum { kElF32 = 0, kElDF = 1, kElF64 = 2 };
+constexpr int kMarchLanes = 8;      // elements of a Nambu row per CTA
+constexpr int march_cols(int el) { return el == kElF32 ? 2 * kMarchLanes : kMarchLanes; }
+constexpr int march_entry_bytes(int el) { return el == kElF32 ? 208 : 400; }  // of a site (13, 25 times 16)
 constexpr int kMarchThreads = 512;  // 16 warps: 128 registers a thread for the 3 x 3 x 2 window and two sums
 // two slabs up to this size stay in L2 (129 MB): 48x24 (85 MB) runs a step in 16.7 us
 // one step per launch, in 25.3 us two, where the halo sites and rows only cost
@@ -151,20 +160,72 @@ __device__ __forceinline__ ulonglong2 march_stencil(const MarchRow<NV>& wm, cons
   return make_ulonglong2(f2sub(a.pr, a.qi), f2add(a.pi, a.qr));
 }
 
+// the same for one complex number per element (C: double-float or FP64), starting
+// from `a` and with the operations of cmac: a site's entries are its two real
+// diagonals (one element), then per component twelve of 16 bytes
+__device__ __forceinline__ float4 el_cast(ulonglong2 u, float4*) {
+  return make_float4(__uint_as_float((unsigned)u.x), __uint_as_float((unsigned)(u.x >> 32)),
+                     __uint_as_float((unsigned)u.y), __uint_as_float((unsigned)(u.y >> 32)));
+}
+__device__ __forceinline__ double2 el_cast(ulonglong2 u, double2*) {
+  return make_double2(__longlong_as_double((long long)u.x), __longlong_as_double((long long)u.y));
+}
+__device__ __forceinline__ ulonglong2 el_bits(float4 v) {
+  return make_ulonglong2((u64)__float_as_uint(v.x) | ((u64)__float_as_uint(v.y) << 32),
+                         (u64)__float_as_uint(v.z) | ((u64)__float_as_uint(v.w) << 32));
+}
+__device__ __forceinline__ ulonglong2 el_bits(double2 v) {
+  return make_ulonglong2((u64)__double_as_longlong(v.x), (u64)__double_as_longlong(v.y));
+}
+template <typename E, int NV, int C, bool HALF>
+__device__ __forceinline__ ulonglong2 march_stencil_el(const MarchRow<NV>& wm, const MarchRow<NV>& w0,
+                                                       const MarchRow<NV>& wp, const E* cq, E a) {
+  E* const tag = nullptr;
+  auto own = [&](const MarchRow<NV>& w, int d) { return el_cast(C ? w.h[d] : w.e[d], tag); };
+  auto oth = [&](const MarchRow<NV>& w, int d) { return el_cast(C ? w.e[d] : w.h[d], tag); };
+  rmac(a, C ? diag1(cq[0]) : diag0(cq[0]), own(w0, 1));
+  const E* c = cq + 1 + 12 * C;
+  auto term = [&](int k, const MarchRow<NV>& w, int d) {
+    const int i = k < 4 ? 2 * k : 8 + (k - 4);
+    cmac(a, c[i], own(w, d));
+    if (k < 4) cmac(a, c[i + 1], oth(w, d));
+  };
+  term(0, w0, 2);
+  term(1, w0, 0);
+  term(2, wp, 1);
+  term(3, wm, 1);
+  term(4, wp, 2);
+  term(5, wm, 0);
+  term(6, wm, 2);
+  term(7, wp, 0);
+  if (HALF) a = vhalf(a);
+  vfinish(a);
+  return el_bits(a);
+}
+
 // where site k of a tile of w <= tx sites sits in a ring row: after the ns sites on its
 // left; the sites on its right follow the full tile's
 __device__ __forceinline__ int march_pos(int k, int w, int tx, int ns) { return k < w ? ns + k : ns + tx + (k - w); }
 // byte offset in a ring row of what slot s of column c of a chunk (own component
-// beta) reads, its site at position p
-template <int NV>
+// beta) reads, its site at position p; and its value in FP64
+template <int EL, int NV>
 __device__ __forceinline__ int march_item(int p, int s, int beta, int c) {
-  return p * 32 * NV + (beta ^ kSlotFlip[s]) * 16 * NV + (c >> 1) * 16 + (c & 1) * 4;
+  return p * 32 * NV + (beta ^ kSlotFlip[s]) * 16 * NV + (EL == kElF32 ? (c >> 1) * 16 + (c & 1) * 4 : c * 16);
+}
+template <int EL>
+__device__ __forceinline__ double2 march_value(const unsigned char* at) {
+  if (EL == kElF64) return *reinterpret_cast<const double2*>(at);
+  const float* e = reinterpret_cast<const float*>(at);
+  if (EL == kElF32) return make_double2((double)e[0], (double)e[2]);
+  return make_double2((double)e[0] + (double)e[1], (double)e[2] + (double)e[3]);
 }
 
-template <int NV, int NS, bool FIRST, bool HOOK>
+template <int EL, int NS, bool FIRST, bool HOOK>
 __global__ void __launch_bounds__(kMarchThreads, 1)
     cheb_march_kernel(const __grid_constant__ MarchMaps vm, const __grid_constant__ MarchMaps pm,
                       const __grid_constant__ MarchArgs a, const __grid_constant__ ColMap cmap) {
+  constexpr int NV = kMarchLanes;
+  constexpr int COLS = march_cols(EL), ENTRYB = march_entry_bytes(EL);
   constexpr int SITE = 2 * NV;         // float4 per site of a row
   constexpr int SITEB = 16 * SITE;     // bytes
   constexpr int LAST = NS - 1;
@@ -186,8 +247,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
   const int nrow = min(ny, y0 + a.ylen) - y0;
   const int x0 = tile * a.tx;
   const int w = min(nx, x0 + a.tx) - x0;
-  const int64_t cb0 = (int64_t)blockIdx.y * (2 * NV);
-  const int64_t q0 = cb0 / 2;
+  const int64_t cb0 = (int64_t)blockIdx.y * COLS;
+  const int64_t q0 = (int64_t)blockIdx.y * NV;
   const int nset = nrow + 2 * LAST;  // rows of stage 0
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -255,7 +316,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     const uint32_t p0 = smem_u32(smem_march), v0 = p0 + vbase, c0 = p0 + cbase;
     const uint32_t vend = p0 + sbase, pend = p0 + vbase, cend = p0 + bbase;
     const uint32_t bytes = rowb + crowb + (FIRST ? 0u : (uint32_t)(full ? nx : a.tx + 2 * LAST) * SITEB);
-    const int col = (int)(2 * cb0), nx2 = 2 * nx;
+    const int col = (int)(4 * q0), nx2 = 2 * nx;
     // a tile's row with the sites around it is one box, or two where it wraps around
     // the lattice: edge = 0 no (or the whole row), 1 on the left, 2 on the right
     const int edge = full ? 0 : x0 == 0 ? 1 : x0 + w == nx ? 2 : 0;
@@ -341,7 +402,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     // chunk's columns whose own site lies in the row and the tile, and arrives beside the stage's warps, which holds the rows it reads
     const bool sums = a.acc != nullptr;
     // unit columns: lane + 32 k is slot (lane + 32 k) % 10 of column (lane + 32 k) / 10
-    constexpr int ITEMS = 2 * NV * kSlots / 32;
+    constexpr int ITEMS = (COLS * kSlots + 31) / 32;
     int iy[ITEMS], off[ITEMS];
     if (sums) {
 #pragma unroll
@@ -350,11 +411,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
         const int64_t col = cmap.s0 + cb0 + c;
         iy[q] = -1;
         off[q] = 0;
-        if (col < (a.D >> cmap.js)) {
+        if (c < COLS && col < (a.D >> cmap.js)) {
           const int J = (int)(col << cmap.js), j = J >> 1;
           const int xj = j % nx, k = xj - x0;
           if (k >= 0 && k < w) iy[q] = j / nx;
-          off[q] = march_item<NV>(full ? wrapi(xj + kSlotDx[sl], nx) : march_pos(k + kSlotDx[sl], w, a.tx, NS), sl,
+          off[q] = march_item<EL, NV>(full ? wrapi(xj + kSlotDx[sl], nx) : march_pos(k + kSlotDx[sl], w, a.tx, NS), sl,
                                   J & 1, c);
         }
       }
@@ -363,7 +424,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     int ylo = ny, yhi = -1;
     double cms[NS], cos[NS];
     if (sums) {
-      const int64_t c0 = cmap.s0 + cb0, c1 = min(a.D >> cmap.js, c0 + 2 * NV) - 1;
+      const int64_t c0 = cmap.s0 + cb0, c1 = min(a.D >> cmap.js, c0 + COLS) - 1;
       if (c1 >= c0) {
         ylo = (int)((c0 << cmap.js) >> 1) / nx;
         yhi = (int)((c1 << cmap.js) >> 1) / nx;
@@ -401,12 +462,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
             if (iy[q] != y) continue;
             const int t = lane + 32 * q, sl = t % kSlots;
             const int64_t J = (cmap.s0 + cb0 + t / kSlots) << cmap.js;
-            const float* e = reinterpret_cast<const float*>(
+            const double2 e = march_value<EL>(
                 smem_march + (kSlotDy[sl] < 0 ? rowat[0] : kSlotDy[sl] > 0 ? rowat[2] : rowat[1]) + off[q]);
-            acc_add_unit(&old[q], sl == kSlots - 1 ? co : cm, (double)e[0], (double)e[2]);
+            acc_add_unit(&old[q], sl == kSlots - 1 ? co : cm, e.x, e.y);
             a.acc[J * kSlots + sl] = old[q];
-            if (sl == 0 && cmap.rec)
-              record_diag(cmap, a.D, a.m + s, J, make_double2(1.0, 0.0), (double)e[0], (double)e[2]);
+            if (sl == 0 && cmap.rec) record_diag(cmap, a.D, a.m + s, J, make_double2(1.0, 0.0), e.x, e.y);
           }
         }
         __syncwarp();
@@ -442,7 +502,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     };
     // the thread's sites x - 1, x, x + 1 in a ring row, its entries
     const int off0 = pos(k - 1) * SITEB + 16 * v, off1 = pos(k) * SITEB + 16 * v, off2 = pos(k + 1) * SITEB + 16 * v;
-    const int ocf = pos(k) * 208;
+    const int ocf = pos(k) * ENTRYB;
     // running positions in the rings of the input, the subtrahend, the output, the entries
     const int inb = st == 0 ? vbase : sbase + (st - 1) * sring, ine = st == 0 ? sbase : inb + sring;
     const int pvb = st == 0 ? 0 : st == 1 ? vbase : sbase + (st - 2) * sring;
@@ -497,21 +557,30 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
         op = op + rowb == pve ? pvb : op + rowb;
         oc = oc + crowb == bbase ? cbase : oc + crowb;
       }
-      float4 q;
-      ulonglong2 o0 = march_stencil<NV, 0>(rm, r0, rp, cq, q);
-      ulonglong2 o1 = march_stencil<NV, 1>(rm, r0, rp, cq, q);
-      if (FIRST && st == 0) {
-        const u64 half2 = 0x3F0000003F000000ull;  // (0.5f, 0.5f)
-        o0.x = f2mul(o0.x, half2);
-        o0.y = f2mul(o0.y, half2);
-        o1.x = f2mul(o1.x, half2);
-        o1.y = f2mul(o1.y, half2);
+      ulonglong2 o0, o1;
+      if constexpr (EL == kElF32) {
+        float4 q;
+        o0 = march_stencil<NV, 0>(rm, r0, rp, cq, q);
+        o1 = march_stencil<NV, 1>(rm, r0, rp, cq, q);
+        if (FIRST && st == 0) {
+          const u64 half2 = 0x3F0000003F000000ull;  // (0.5f, 0.5f)
+          o0.x = f2mul(o0.x, half2);
+          o0.y = f2mul(o0.y, half2);
+          o1.x = f2mul(o1.x, half2);
+          o1.y = f2mul(o1.y, half2);
+        } else {
+          const ulonglong2 b0 = ld16(p), b1 = ld16(p + hd);
+          o0.x = f2sub(o0.x, b0.x);
+          o0.y = f2sub(o0.y, b0.y);
+          o1.x = f2sub(o1.x, b1.x);
+          o1.y = f2sub(o1.y, b1.y);
+        }
       } else {
-        const ulonglong2 b0 = ld16(p), b1 = ld16(p + hd);
-        o0.x = f2sub(o0.x, b0.x);
-        o0.y = f2sub(o0.y, b0.y);
-        o1.x = f2sub(o1.x, b1.x);
-        o1.y = f2sub(o1.y, b1.y);
+        using E = std::conditional_t<EL == kElDF, float4, double2>;
+        E* const tag = nullptr;
+        const E* ce = reinterpret_cast<const E*>(cq);
+        o0 = march_stencil_el<E, NV, 0, FIRST>(rm, r0, rp, ce, FIRST ? vzero<E>() : vneg(el_cast(ld16(p), tag)));
+        o1 = march_stencil_el<E, NV, 1, FIRST>(rm, r0, rp, ce, FIRST ? vzero<E>() : vneg(el_cast(ld16(p + hd), tag)));
       }
       if (NS > 1 && st < LAST) {
         if (on) {

@@ -254,8 +254,8 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
     if (pp->ranged && (o->flags & KPM_FLAG_PH_HALF))
       return fail(ctx, KPM_EINVAL, "KPM_FLAG_PH_HALF and a site range do not combine");
   }
-  const bool march = o->precision == KPM_FP32;
-  const bool deeper = march && pp_ == 0 && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
+  const bool march = o->precision == KPM_FP32 || pp_ == 0;  // (FP64 and double-float probing: the one-step kernels)
+  const bool deeper = o->precision == KPM_FP32 && pp_ == 0 && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
   const int js = (o->flags & KPM_FLAG_PH_HALF) ? 1 : 0;
   // start vectors of the pass: unit columns (those of the site range), or R = 2 p^2 probing vectors
   pp->c0 = pp->ranged ? 2 * (int64_t)pp->sb : 0;
@@ -269,7 +269,7 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
     return balanced_width(ncols, std::min<int64_t>(ncols, std::max<int64_t>(fit, 1)));
   };
   int64_t width = width_of(2);
-  int steps = march ? (single || pp_ > 0 ? 1 : march_steps(m->nx, m->ny, width)) : 0;
+  int steps = march ? (single || pp_ > 0 || o->precision != KPM_FP32 ? 1 : march_steps(m->nx, m->ny, width)) : 0;
   if (steps > 1 && (o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
   if (deeper) ++steps;
   if (steps > 1) width = width_of(4);
@@ -278,7 +278,7 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
   pp->cheb.js = js;
   pp->cheb.probe_p = pp_;
   pp->cheb.probe_seed = (uint32_t)o->probe_seed;
-  pp->cheb.raw = march && pp_ > 0 && o->M >= 2;
+  pp->cheb.raw = o->precision == KPM_FP32 && pp_ > 0 && o->M >= 2;
   if (pp->cheb.cb == 0) return fail(ctx, KPM_EINVAL, "lattice row too wide for the shared-memory window");
   // slabs advance by the padded width: every unit column belongs to exactly one slab
   pp->width = pp->cheb.ldv;
@@ -314,7 +314,7 @@ int ensure_pass_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, con
     if (ctx->xi_bytes < (size_t)D * sizeof(double2)) drop_graph(ctx);
     if ((r = ensure(ctx, &ctx->xi, &ctx->xi_bytes, (size_t)D * sizeof(double2)))) return r;
   }
-  // FP32 unit vectors: the entries in the ring rows' layout of both launch plans
+  // march kernel: the entries in the ring rows' layout of both launch plans
   const size_t tb = pp.cheb.mk.ns ? march_table_bytes(pp.cheb.mk, m->ny) + march_table_bytes(pp.cheb.m1, m->ny)
                                   : (size_t)m->nx * m->ny * table_bytes_per_site(o->precision);
   if (ctx->table_bytes < tb) drop_graph(ctx);
@@ -1017,10 +1017,7 @@ int kpm_backward(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
   void* A = ctx->slab[0];
   void* B = ctx->slab[1];
   KPM_CU(launch_coefficients(M, ab, ctx->am, ctx->ao, s, 0, o.temperature));
-  if (prec == KPM_FP32)
-    KPM_CU(launch_march_table(*model, p.m1, fields, ab, (float4*)ctx->table, s));
-  else
-    KPM_CU(launch_scale_table_f64(*model, fields, ab, (double2*)ctx->table, s));
+  KPM_CU(launch_march_table(*model, p.m1, fields, ab, (float4*)ctx->table, s));
   // seeds of the columns outside the site range are zero: their backward
   // vectors stay zero, so they add nothing where a slab runs past the range
   KPM_CU(launch_seed_weights(model->nx, model->ny, grad_obs, ab, grad_omega, ctx->wseed, s, pp.sb, pp.se));
@@ -1261,8 +1258,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   // per-cell scratch, one allocation per cell
   auto al = [](size_t n) { return (n + 255) & ~(size_t)255; };
   auto tab_bytes = [&](int k, int N) {
-    return prec == KPM_FP32 && !persist[k] ? march_table_bytes(plans[k].m1, plans[k].ny)
-                                           : (size_t)N * table_bytes_per_site(prec);
+    return persist[k] ? (size_t)N * table_bytes_per_site(prec) : march_table_bytes(plans[k].m1, plans[k].ny);
   };
   bool realloc = (int)ctx->cells.size() != ncell;
   std::vector<size_t> need(ncell);
@@ -1430,10 +1426,8 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
       KPM_TRY(launch_coefficients(M, C.misc, C.am, C.ao, c0, 0, opts->temperature));
       if (prec == KPM_FP32 && persist[C.cls])
         KPM_TRY(launch_scale_table_f32(m, C.fields, C.misc, (float2*)C.table, c0));
-      else if (prec == KPM_FP32)
-        KPM_TRY(launch_march_table(m, p.m1, C.fields, C.misc, (float4*)C.table, c0));
       else
-        KPM_TRY(launch_scale_table_f64(m, C.fields, C.misc, (double2*)C.table, c0));
+        KPM_TRY(launch_march_table(m, p.m1, C.fields, C.misc, (float4*)C.table, c0));
       if (!persist[C.cls]) KPM_TRY(launch_cheb_init(p, prec, C.A, 0, C.acc, C.am, C.ao, c0));
     }
     // recursion: one chain per shape class on its own stream

@@ -14,9 +14,10 @@ constexpr int kSlots = 10;     // accumulated entries per unit column (9 local r
 constexpr int kCoef = 26;      // complex 2h~ entries per site (both Nambu rows, padded)
 constexpr int kRedBlock = 256; // threads of the reduction kernels
 
-// Launch geometry of the FP32 march kernel (ns recursion steps per launch).
+// Launch geometry of the march kernel (ns recursion steps per launch).
 struct MarchPlan {
   int ns = 0;                  // steps per launch (0: not planned)
+  int el = 0;                  // element: 0 FP32 column pairs, 1 double-float, 2 FP64
   int tx = 0, ntile = 0, full = 0;  // sites per tile, tiles per lattice row, one tile covers the row
   int ylen = 0;                // lattice rows per band
   int wrow = 0, crowb = 0;     // sites of a ring row, bytes of its entries
@@ -31,7 +32,7 @@ struct alignas(64) SlabMaps {
 
 // Launch geometry of the recursion kernel (shared with the host planner).
 struct ChebPlan {
-  MarchPlan mk;    // FP32: the pass's launches of several steps (or one)
+  MarchPlan mk;    // march kernel: the pass's launches of several steps (or one)
   MarchPlan m1;    // and the single step
   int nx, ny;
   int64_t D;       // 2 N
@@ -125,8 +126,8 @@ cudaError_t launch_update(int N, double* params, double* obs, double* mu_eff, co
 int reduce_scratch_doubles(int64_t n);
 
 // ---------------------------------------------------------------- cheb_kernels.cu
-// steps: FP32 recursion steps per launch of the march kernel (chunks of 16 columns);
-// 0: the one-step kernels (FP64, double-float, narrower FP32 chunks)
+// steps: recursion steps per launch of the march kernel (FP64 and double-float: one;
+// chunks of 16 FP32 columns or 8); 0: the one-step kernels with their narrower chunks
 ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0, int steps = 0);
 // FP32 steps per launch at which unit-vector slabs of `width` columns run fastest
 int march_steps(int nx, int ny, int64_t width);
@@ -148,7 +149,7 @@ cudaError_t launch_cheb_init(const ChebPlan& p, int precision, void* V0, int64_t
 cudaError_t launch_cheb_step(const ChebPlan& p, int precision, const void* table, const void* Vcur,
                              void* Vout, int64_t s0, double2* acc, const double* am,
                              const double* ao, int m, int mode, cudaStream_t s, const void* Vprev = nullptr);
-// device fault word of the FP32 march kernel (bit 0: a bounded wait
+// device fault word of the march kernel (bit 0: a bounded wait
 // expired; bit 1: shared memory misaligned for TMA); sticky for the process
 cudaError_t read_step_fault(unsigned int* out);
 cudaError_t clear_step_fault();

@@ -99,13 +99,13 @@ extern "C" int kpm_observables_noalloc(const kpm_model* m, const kpm_opts* o, co
   const size_t off_ao = align256(off_am + (size_t)o->M * sizeof(double));
   const size_t off_red = align256(off_ao + (size_t)o->M * sizeof(double));
   const size_t off_tab = align256(off_red + (size_t)reduce_scratch_doubles(0) * sizeof(double));
-  // widest slab (unit columns per recursion) whose two buffers fit the rest: FP32 by
-  // the march kernel, or, where its 16-column chunk does not fit, by the narrower
-  // chunks of the one-step kernels
+  // widest slab (unit columns per recursion) whose two buffers fit the rest: by the
+  // march kernel, or, where its chunk does not fit, by the narrower chunks of the
+  // one-step kernels
   size_t off_acc = 0, off_slab = 0;
   ChebPlan p;
   int64_t width = 0;
-  for (int steps = o->precision == KPM_FP32 ? 1 : 0; steps >= 0; --steps) {
+  for (int steps = 1; steps >= 0; --steps) {
     p = plan_cheb(m->nx, m->ny, D, o->precision, o->cols_per_block, o->band_rows, steps);
     if (p.cb == 0) return KPM_EINVAL;
     off_acc = align256(off_tab + (p.m1.ns ? march_table_bytes(p.m1, m->ny) : (size_t)N * table_bytes_per_site(o->precision)));

@@ -528,10 +528,12 @@ __global__ void scale_table_kernel(kpm_model m, const double* __restrict__ fld, 
   for (int k = 0; k < kCoef; ++k) out[k] = e[k];
 }
 
-// the entries in the order in which the march kernel's sums use them: for each
-// component the diagonal, then per neighbour its hop and (first four) its pairing
-// (25 floats each, 52 with padding), for the sites of every tile's ring row: halo
-// sites on its left, its own (tx, fewer in the last tile), halo sites on its right
+// the entries in the order in which the march kernel's sums use them, for the sites of
+// every tile's ring row: halo sites on its left, its own (tx, fewer in the last
+// tile), halo sites on its right.  FP32: for each component the diagonal, then per
+// neighbour its hop and (first four) its pairing (25 floats each, 52 with padding);
+// double-float and FP64: both diagonals as one element, then the same 12 per component.
+template <typename C>
 __global__ void march_table_kernel(kpm_model m, const double* __restrict__ fld, const double* __restrict__ ab,
                                    float4* __restrict__ table, int tx, int ntile, int wrow, int crow, int halo) {
   const int at = blockIdx.x * blockDim.x + threadIdx.x;
@@ -542,31 +544,44 @@ __global__ void march_table_kernel(kpm_model m, const double* __restrict__ fld, 
   if (p >= halo + tx) k = w + (p - halo - tx);
   else if (k >= w) k = w - 1;  // no site: any
   const int x = (x0 + k + m.nx) % m.nx, i = y * m.nx + x;
-  float2 e[kCoef];
-  site_entries<float2>(m, fld, ab, i, e);
-  float o[2 * kCoef];
+  C e[kCoef];
+  site_entries<C>(m, fld, ab, i, e);
+  float4* const row = table + (size_t)(at / wrow) * crow;
+  if constexpr (sizeof(C) == 8) {
+    float o[2 * kCoef];
 #pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const bool up = c == 0;
-    float* q = o + 25 * c;
-    q[0] = up ? e[0].x : e[0].y;
+    for (int c = 0; c < 2; ++c) {
+      float* q = o + 25 * c;
+      q[0] = c == 0 ? e[0].x : e[0].y;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int to = k < 4 ? 1 + 4 * k : 17 + 2 * (k - 4);
-      const float2 hop = up ? e[1 + k] : e[9 + k];
-      q[to] = hop.x;
-      q[to + 1] = hop.y;
-      if (k < 4) {
-        const float2 pair = up ? e[17 + k] : e[21 + k];
-        q[to + 2] = pair.x;
-        q[to + 3] = pair.y;
+      for (int n = 0; n < 8; ++n) {
+        const int to = n < 4 ? 1 + 4 * n : 17 + 2 * (n - 4);
+        const C hop = e[(c == 0 ? 1 : 9) + n];
+        q[to] = hop.x;
+        q[to + 1] = hop.y;
+        if (n < 4) {
+          const C pair = e[(c == 0 ? 17 : 21) + n];
+          q[to + 2] = pair.x;
+          q[to + 3] = pair.y;
+        }
       }
     }
-  }
-  o[50] = o[51] = 0.f;
-  float4* out = table + (size_t)(at / wrow) * crow + p * (kCoef / 2);
+    o[50] = o[51] = 0.f;
+    float4* out = row + p * (kCoef / 2);
 #pragma unroll
-  for (int k = 0; k < kCoef / 2; ++k) out[k] = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+    for (int n = 0; n < kCoef / 2; ++n) out[n] = make_float4(o[4 * n], o[4 * n + 1], o[4 * n + 2], o[4 * n + 3]);
+  } else {
+    C* out = reinterpret_cast<C*>(row) + p * 25;
+    out[0] = e[0];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int n = 0; n < 8; ++n) {
+        const int to = 1 + 12 * c + (n < 4 ? 2 * n : 8 + (n - 4));
+        out[to] = e[(c == 0 ? 1 : 9) + n];
+        if (n < 4) out[to + 1] = e[(c == 0 ? 17 : 21) + n];
+      }
+  }
 }
 
 // Observables from the accumulated entries of F_M(h~) e_J (readings N2, N3):
@@ -1075,8 +1090,9 @@ cudaError_t launch_scale_table_f32(const kpm_model& m, const double* fields, con
 cudaError_t launch_march_table(const kpm_model& m, const MarchPlan& mp, const double* fields, const double* ab,
                                float4* table, cudaStream_t s) {
   const int n = m.ny * mp.ntile * mp.wrow;
-  march_table_kernel<<<(n + 127) / 128, 128, 0, s>>>(m, fields, ab, table, mp.tx, mp.ntile, mp.wrow,
-                                                      mp.crowb / 16, mp.full ? 0 : mp.ns);
+  auto fn = mp.el == 0 ? march_table_kernel<float2> : mp.el == 1 ? march_table_kernel<float4> : march_table_kernel<double2>;
+  fn<<<(n + 127) / 128, 128, 0, s>>>(m, fields, ab, table, mp.tx, mp.ntile, mp.wrow, mp.crowb / 16,
+                                     mp.full ? 0 : mp.ns);
   return cudaGetLastError();
 }
 

@@ -110,3 +110,19 @@ def test_probing_sums_of_every_order(K, nx, ny, p, bw, M):
     cell = _cell(K, nx, ny)
     kw = dict(block_width=bw, probe_p=p, probe_seed=3)
     assert np.max(np.abs(_pass(K, cell, M, 1, **kw)[:-1] - _pass(K, cell, M, 0, **kw)[:-1])) < 2e-5
+
+
+@pytest.mark.parametrize("nx,ny", [(2, 2), (3, 5), (29, 4), (56, 3), (57, 4), (113, 2)])
+@pytest.mark.parametrize("M", [2, 3, 9])
+@pytest.mark.parametrize("prec", ["fp64", "df64"])
+def test_fp64_and_double_float_plans(K, nx, ny, M, prec):
+    """FP64 and double-float on the march kernel: the same bits for every band and slab, within
+    1e-10 of the FP64 pass (double-float: about 48 bits, at most 9 steps of growth)."""
+    kpm, _ = K
+    P = kpm.KPM_FP64 if prec == "fp64" else kpm.KPM_DF64
+    cell = _cell(K, nx, ny)
+    ref = _pass(K, cell, M, P)
+    for kw in (dict(band_rows=1), dict(band_rows=max(1, ny - 1)), dict(block_width=24, band_rows=2)):
+        got = _pass(K, cell, M, P, **kw)
+        assert np.array_equal(got[:-1], ref[:-1]), kw
+    assert np.max(np.abs(_pass(K, cell, M, kpm.KPM_FP64)[:-1] - ref[:-1])) < 1e-10
