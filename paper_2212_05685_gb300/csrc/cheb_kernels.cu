@@ -15,8 +15,8 @@
 // Layout: V is row-major, V[K][c] with K = 2 i + alpha the Nambu row and c the
 // column inside the slab; the row stride ldv is the slab width rounded up to
 // the CTA's column chunk.  FP64 stores interleaved complex (re, im);
-// double-float (KPM_DF64) stores (re_hi, re_lo, im_hi, im_lo), each real the
-// unevaluated FP32 sum hi + lo, and runs the FP64 kernel's structure with
+// double-float (KPM_DF64) stores (re_hi, im_hi, re_lo, im_lo), each real the
+// unevaluated FP32 sum hi + lo, so that a packed f32x2 operation works on both, and runs the FP64 kernel's structure with
 // double-float arithmetic.  FP32 stores each column pair (2p, 2p+1) as
 // (re_2p, re_2p+1, im_2p, im_2p+1) so that one packed f32x2 FMA advances two
 // columns.  h~ is a 13-point stencil per row (diagonal, eight hops, four
@@ -88,8 +88,8 @@ __device__ __forceinline__ double cim(double2 v) { return v.y; }
 
 // Double-float (KPM_DF64): every real is the unevaluated sum hi + lo of two
 // FP32 numbers, about 48 significant bits, so the FP64-accurate recursion runs
-// on the FP32 pipes.  A complex element is float4 (re_hi, re_lo, im_hi, im_lo);
-// table entry 0 holds the two real diagonals as (d0_hi, d0_lo, d1_hi, d1_lo).
+// on the FP32 pipes.  A complex element of a vector is float4 (re_hi, im_hi, re_lo,
+// im_lo), of the table (re_hi, re_lo, im_hi, im_lo); table entry 0 holds the two real diagonals as (d0_hi, d0_lo, d1_hi, d1_lo).
 // Products use the exact FMA residual of hi * hi (p + e = xh yh exactly) plus
 // the cross terms; sums use Knuth's two-sum, whose error term is exact for any
 // ordering of the operands; an accumulator is renormalised once per output.
@@ -117,14 +117,14 @@ __device__ __forceinline__ void df_mac(float& h, float& l, float xh, float xl, f
   l = __fadd_rn(l, __fadd_rn(t, e));
 }
 __device__ __forceinline__ void cmac(float4& a, float4 c, float4 v) {
-  df_mac(a.x, a.y, c.x, c.y, v.x, v.y);
-  df_mac(a.x, a.y, -c.z, -c.w, v.z, v.w);
-  df_mac(a.z, a.w, c.x, c.y, v.z, v.w);
-  df_mac(a.z, a.w, c.z, c.w, v.x, v.y);
+  df_mac(a.x, a.z, c.x, c.y, v.x, v.z);
+  df_mac(a.x, a.z, -c.z, -c.w, v.y, v.w);
+  df_mac(a.y, a.w, c.x, c.y, v.y, v.w);
+  df_mac(a.y, a.w, c.z, c.w, v.x, v.z);
 }
 __device__ __forceinline__ void rmac(float4& a, float2 d, float4 v) {
-  df_mac(a.x, a.y, d.x, d.y, v.x, v.y);
-  df_mac(a.z, a.w, d.x, d.y, v.z, v.w);
+  df_mac(a.x, a.z, d.x, d.y, v.x, v.z);
+  df_mac(a.y, a.w, d.x, d.y, v.y, v.w);
 }
 __device__ __forceinline__ float4 vneg(float4 v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
 __device__ __forceinline__ float4 vhalf(float4 v) { return make_float4(0.5f * v.x, 0.5f * v.y, 0.5f * v.z, 0.5f * v.w); }
@@ -132,17 +132,17 @@ template <>
 __device__ __forceinline__ float4 vzero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 __device__ __forceinline__ void vfinish(float4& v) {
   float h, l;
-  two_sum(v.x, v.y, h, l);
+  two_sum(v.x, v.z, h, l);
   v.x = h;
-  v.y = l;
-  two_sum(v.z, v.w, h, l);
-  v.z = h;
+  v.z = l;
+  two_sum(v.y, v.w, h, l);
+  v.y = h;
   v.w = l;
 }
 __device__ __forceinline__ float2 diag0(float4 d) { return make_float2(d.x, d.y); }
 __device__ __forceinline__ float2 diag1(float4 d) { return make_float2(d.z, d.w); }
-__device__ __forceinline__ double cre(float4 v) { return (double)v.x + (double)v.y; }
-__device__ __forceinline__ double cim(float4 v) { return (double)v.z + (double)v.w; }
+__device__ __forceinline__ double cre(float4 v) { return (double)v.x + (double)v.z; }
+__device__ __forceinline__ double cim(float4 v) { return (double)v.y + (double)v.w; }
 // FP64 value as hi + lo (the rounding residual of hi is exact in FP64)
 __device__ __forceinline__ float2 df_split(double x) {
   const float h = __double2float_rn(x);
@@ -843,7 +843,7 @@ __global__ void cheb_init_df_kernel(int64_t D, int64_t ldv, int nx, float4* __re
     const int64_t K = k / ldv, c = k - K * ldv;
     const double2 e = start_entry(K, c, D, nx, cm);
     const float2 re = df_split(e.x), im = df_split(e.y);
-    V0[k] = make_float4(re.x, re.y, im.x, im.y);
+    V0[k] = make_float4(re.x, im.x, re.y, im.y);
   }
 }
 // FP32 pair-split layout: float4 (re_2p, re_2p+1, im_2p, im_2p+1)
