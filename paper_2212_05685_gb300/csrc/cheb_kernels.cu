@@ -1396,8 +1396,11 @@ namespace {
 // band heights of a march launch: as many CTAs per SM as registers and shared memory
 // take; a CTA's start (barriers, first copies) costs about five rows (one of double-float
 // or FP64), and a launch of several steps computes two more rows for every step but the last
+int march_per_sm(const MarchPlan& p) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(16 / p.warps, (int64_t)(228 * 1024) / (int64_t)(p.smem + 1024)));
+}
 int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
-  const int per_sm = (int)std::max<int64_t>(1, std::min<int64_t>(16 / p.warps, (int64_t)(228 * 1024) / (int64_t)(p.smem + 1024)));
+  const int per_sm = march_per_sm(p);
   const double start = p.el == kElF32 ? 5.0 + 2.0 * (p.ns - 1) : 1.0;
   return band_rows_candidates(ny, ldv / march_cols(p.el) * p.ntile, out, maxn, per_sm * kSMs, start);
 }
@@ -1488,7 +1491,7 @@ size_t march_table_bytes(const MarchPlan& mp, int ny) { return (size_t)mp.crowb 
 
 cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* table, const SlabMaps& cur,
                          const SlabMaps& prev, void* outa, void* outb, int64_t s0, double2* acc, const double* am,
-                         const double* ao, int m, bool first, cudaStream_t s) {
+                         const double* ao, int m, bool first, cudaStream_t s, int64_t col0, int64_t cols) {
   MarchArgs a;
   a.nx = p.nx;
   a.ny = p.ny;
@@ -1513,11 +1516,12 @@ cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* tab
   a.am = am;
   a.ao = ao;
   a.m = m;
+  a.chunk0 = (int)(col0 / march_cols(mp.el));
   a.grow = 16 * 2 * (int64_t)p.nx * a.ldq;
   MarchMaps v, pr;
   memcpy(&v, cur.v, sizeof(v));
   memcpy(&pr, prev.p, sizeof(pr));
-  const dim3 grid((unsigned)(((p.ny + mp.ylen - 1) / mp.ylen) * mp.ntile), (unsigned)(p.ldv / march_cols(mp.el)));
+  const dim3 grid((unsigned)(((p.ny + mp.ylen - 1) / mp.ylen) * mp.ntile), (unsigned)((cols > 0 ? std::min(cols, p.ldv - col0) : p.ldv) / march_cols(mp.el)));
   const ColMap cm = colmap(p, s0);
   if (mp.el == kElDF) return march_launch<kElDF, 1>(mp, grid, v, pr, a, cm, first, s);
   if (mp.el == kElF64) return march_launch<kElF64, 1>(mp, grid, v, pr, a, cm, first, s);
@@ -1549,7 +1553,8 @@ int band_rows_candidates(int ny, int64_t ctas, int* out, int maxn, int slots, do
   return n;
 }
 
-ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request, int band_rows, int steps) {
+ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request, int band_rows, int steps,
+                   bool split) {
   ChebPlan p;
   p.nx = nx;
   p.ny = ny;
@@ -1557,6 +1562,7 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
   p.nthreads = 512;
   p.cb = 0;
   p.ldv = 0;
+  p.sub = 0;
   p.smem = 0;
   p.ylen = ny;
   p.js = 0;
@@ -1592,7 +1598,8 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
     const int el = precision == KPM_FP32 ? kElF32 : precision == KPM_DF64 ? kElDF : kElF64;
     p.cb = march_cols(el);
     p.ldv = (width + p.cb - 1) / p.cb * p.cb;
-    p.m1 = plan_march(nx, ny, p.ldv, 1, band_rows, el);
+    p.sub = split && steps == 1 && el == kElF32 ? march_columns(nx, ny, p.ldv) : p.ldv;
+    p.m1 = plan_march(nx, ny, p.sub, 1, band_rows, el);
     p.mk = steps > 1 && el == kElF32 ? plan_march(nx, ny, p.ldv, steps, band_rows) : p.m1;
     if (p.mk.ns == 0) p.mk = p.m1;
     p.ylen = p.mk.ylen;
@@ -1612,18 +1619,59 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
 }
 
 
+namespace {
+// us per step of single steps over the cheapest number of parts of a slab (*cols columns).
+// Above L2 the single steps of a whole slab run at the memory's rate (6.3 TB/s of copies).
+// Parts that fit L2 do not, but pay the launches' starts, and a part's CTAs fill the SMs
+// more or less well: rows of 0.0485 us per stage warp (48x24, 64x32, 64x64: the same within
+// 5%).  Measured, whole slab against parts: 40x40 45.9 -> 39 (3 parts), 64x32 75 -> 61 (4),
+// 64x64 257 -> 217 (14); up to sixteen parts, beyond which launches only add up
+// (80x80 603 -> 601, 27 parts).
+double parts_us(int nx, int ny, int64_t width, int64_t* cols) {
+  const int64_t D = 2 * (int64_t)nx * ny, cb = march_cols(kElF32), chunks = (width + cb - 1) / cb;
+  *cols = chunks * cb;
+  double cost = 24.0 * (double)D * (double)width / 6.3e6;
+  const MarchPlan p = plan_march(nx, ny, width, 1, 0);
+  if (p.ns == 0 || 16 * D * width <= kMarchL2) return cost;
+  const int per_sm = march_per_sm(p);
+  const double row_us = 0.0485 * (p.warps - 2) * per_sm;
+  for (int n = 2; n <= 16 && n <= chunks; ++n) {
+    const int64_t c = (chunks + n - 1) / n;
+    if (16 * D * cb * c > kMarchL2) continue;
+    int rows = ny;
+    march_bands(p, ny, c * cb, &rows, 1);
+    const int64_t ctas = c * p.ntile * ((ny + rows - 1) / rows);
+    const double us = n * row_us * (rows + 5.0) * (double)((ctas + per_sm * kSMs - 1) / (per_sm * kSMs));
+    if (us < cost) {
+      cost = us;
+      *cols = c * cb;
+    }
+  }
+  return cost;
+}
+}  // namespace
+
 // Two steps per launch where the slabs stream from memory and the tile fills its
 // warps: 100x100 (13 or 14 stage warps) 1248 against 1457 us per step, a 2500-column
-// slab of it 180 against 213; 64x64, whose tiles of 22 sites fill 11.5, 275 against 266
+// slab of it 180 against 213; 64x64, whose tiles of 22 sites fill 11.5, 275 against 266.
+// Not where parts that fit L2 are cheaper than its 3.3 ps per row-column (60x60 to
+// 100x100: 3.1 to 3.4; 48x48, 3.75: 79.7 against 70 us in four parts).
 int march_steps(int nx, int ny, int64_t width) {
   const int64_t D = 2 * (int64_t)nx * ny;
   if (16 * D * width <= kMarchL2) return 1;
   const MarchPlan p = plan_march(nx, ny, width, 2, 0);
-  return p.ns == 2 && p.warps >= 15 ? 2 : 1;
+  int64_t cols;
+  return p.ns == 2 && p.warps >= 15 && 3.3e-6 * (double)D * (double)width < parts_us(nx, ny, width, &cols) ? 2 : 1;
+}
+
+int64_t march_columns(int nx, int ny, int64_t width) {
+  int64_t cols;
+  parts_us(nx, ny, width, &cols);
+  return cols;
 }
 
 int plan_band_candidates(const ChebPlan& p, int* out, int maxn) {
-  if (p.mk.ns) return march_bands(p.mk, p.ny, p.ldv, out, maxn);
+  if (p.mk.ns) return march_bands(p.mk, p.ny, p.mk.ns == 1 ? p.sub : p.ldv, out, maxn);
   return band_rows_candidates(p.ny, p.ldv / p.cb, out, maxn);
 }
 

@@ -57,8 +57,8 @@ constexpr int kMarchLanes = 8;      // elements of a Nambu row per CTA
 constexpr int march_cols(int el) { return el == kElF32 ? 2 * kMarchLanes : kMarchLanes; }
 constexpr int march_entry_bytes(int el) { return el == kElF32 ? 208 : 400; }  // of a site (13, 25 times 16)
 constexpr int kMarchThreads = 512;  // 16 warps: 128 registers a thread for the 3 x 3 x 2 window and two sums
-// two slabs up to this size stay in L2 (129 MB): 48x24 (85 MB) runs a step in 16.7 us
-// one step per launch, in 25.3 us two, where the halo sites and rows only cost
+// what two slabs touch stays in L2 (129 MB) up to this size: 48x24 (85 MB) runs a step in
+// 16.7 us one step per launch, in 25.3 us two, where the halo sites and rows only cost
 constexpr int64_t kMarchL2 = 100000000;
 constexpr int kMarchBars = 16;      // phases of every barrier ring
 constexpr int kMarchRows = 8;       // rows of every ring of a launch of several steps
@@ -84,6 +84,7 @@ struct MarchArgs {
   const double* am;
   const double* ao;
   int m;
+  int chunk0;           // the launch's first column chunk
   int64_t grow;         // bytes of a lattice row of a slab
 };
 
@@ -302,8 +303,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
   const int nrow = min(ny, y0 + a.ylen) - y0;
   const int x0 = tile * a.tx;
   const int w = min(nx, x0 + a.tx) - x0;
-  const int64_t cb0 = (int64_t)blockIdx.y * COLS;
-  const int64_t q0 = (int64_t)blockIdx.y * NV;
+  const int64_t cb0 = (int64_t)(a.chunk0 + blockIdx.y) * COLS;
+  const int64_t q0 = (int64_t)(a.chunk0 + blockIdx.y) * NV;
   const int nset = nrow + 2 * LAST;  // rows of stage 0
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;

@@ -273,7 +273,8 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
   if (steps > 1 && (o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
   if (deeper) ++steps;
   if (steps > 1) width = width_of(4);
-  pp->cheb = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows, steps);
+  pp->cheb = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows, steps,
+                       !single && pp_ == 0);
   pp->deeper = deeper && pp->cheb.mk.ns == steps;
   pp->cheb.js = js;
   pp->cheb.probe_p = pp_;
@@ -388,6 +389,20 @@ int enqueue_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, const Pass
     KPM_CU(launch_cheb_init(p, prec, ctx->slab[0], s0, ctx->acc, ctx->am, ctx->ao, s));
     nl += 1;
     if (events && s0 == pp.c0) KPM_CU(cudaEventRecordWithFlags(ctx->ev[0], s, cudaEventRecordExternal));
+    // a single step per launch: part of the columns after part, each through all its steps
+    for (int64_t col = 0; p.mk.ns == 1 && p.sub < p.ldv && col < p.ldv; col += p.sub) {
+      const double part = (double)std::min(p.sub, p.ldv - col) / (double)p.ldv;
+      ix = iy = 0;
+      for (mm = 0; mm < M - 1; ++mm) {
+        const int io = mm == 0 ? 1 : ix;
+        KPM_CU(launch_march(p, p.m1, table1, m1[iy], m1[ix], nullptr, ctx->slab[io], s0, ctx->acc, ctx->am, ctx->ao,
+                            mm, mm == 0, s, col, p.sub));
+        nb += (mm == 0 ? 2 : 3) * vec * part;
+        ix = iy;
+        iy = io;
+        nr += 1;
+      }
+    }
     while (mm < M - 1) {
       const bool first = mm == 0;
       if (p.mk.ns > 1 && mm + p.mk.ns <= M - 1) {

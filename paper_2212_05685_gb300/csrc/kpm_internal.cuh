@@ -34,6 +34,7 @@ struct alignas(64) SlabMaps {
 struct ChebPlan {
   MarchPlan mk;    // march kernel: the pass's launches of several steps (or one)
   MarchPlan m1;    // and the single step
+  int64_t sub;     // columns of a single-step launch of a unit-vector pass, which run all their steps in turn
   int nx, ny;
   int64_t D;       // 2 N
   int64_t ldv;     // slab width padded to a multiple of cb (complex elements per row)
@@ -127,10 +128,14 @@ int reduce_scratch_doubles(int64_t n);
 
 // ---------------------------------------------------------------- cheb_kernels.cu
 // steps: recursion steps per launch of the march kernel (FP64 and double-float: one;
-// chunks of 16 FP32 columns or 8); 0: the one-step kernels with their narrower chunks
-ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0, int steps = 0);
+// chunks of 16 FP32 columns or 8); 0: the one-step kernels with their narrower chunks.
+// split: FP32 single steps over parts of the slab (march_columns)
+ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0, int steps = 0,
+                   bool split = false);
 // FP32 steps per launch at which unit-vector slabs of `width` columns run fastest
 int march_steps(int nx, int ny, int64_t width);
+// and the columns of a slab of `width` that run all their single steps before the next ones
+int64_t march_columns(int nx, int ny, int64_t width);
 // up to maxn band heights (lattice rows per CTA) for `ctas` CTAs per band of an
 // ny-row lattice, best first by a wave model: `slots` CTAs run at a time, each
 // costing its rows and `extra` more
@@ -164,7 +169,7 @@ cudaError_t encode_slab_maps(const ChebPlan& p, const MarchPlan& mp, const void*
                              bool as_p = true);
 cudaError_t launch_march(const ChebPlan& p, const MarchPlan& mp, const void* table, const SlabMaps& cur,
                          const SlabMaps& prev, void* outa, void* outb, int64_t s0, double2* acc, const double* am,
-                         const double* ao, int m, bool first, cudaStream_t s);
+                         const double* ao, int m, bool first, cudaStream_t s, int64_t col0 = 0, int64_t cols = 0);
 size_t march_table_bytes(const MarchPlan& mp, int ny);
 // table conj(xi_J) of the probing phases, J < D
 cudaError_t launch_probe_phases(const ChebPlan& p, double2* xi_conj, cudaStream_t s);

@@ -126,3 +126,19 @@ def test_fp64_and_double_float_plans(K, nx, ny, M, prec):
         got = _pass(K, cell, M, P, **kw)
         assert np.array_equal(got[:-1], ref[:-1]), kw
     assert np.max(np.abs(_pass(K, cell, M, kpm.KPM_FP64)[:-1] - ref[:-1])) < 1e-10
+
+
+@pytest.mark.parametrize("nx,ny", [(40, 40), (48, 48), (64, 32), (41, 43), (20, 128), (64, 64)])
+def test_parts_of_a_slab_equal_slabs(K, nx, ny):
+    """Slabs above L2 that run part after part through all their steps, against narrow slabs, whose
+    launches have no parts."""
+    cell = _cell(K, nx, ny)
+    M = 8
+    parts = _pass(K, cell, M)
+    slabs = _pass(K, cell, M, block_width=400)
+    assert np.array_equal(parts[:-1], slabs[:-1])
+    N = nx * ny
+    lo, hi = N // 7, N - 3
+    part = _pass(K, cell, M, site_begin=lo, site_end=hi)
+    assert np.array_equal(part[lo:hi], slabs[lo:hi])
+    assert not part[:lo].any() and not part[hi:N].any()
