@@ -105,7 +105,10 @@ struct kpm_ctx {
   size_t pbuf_bytes = 0;
   cudaEvent_t pev[2] = {nullptr, nullptr};
   int p_launched = 0;              // 1 when the captured batch graph holds the persistent launch
-  double p_bytes = 0;              // its streaming-equivalent bytes per iteration
+  double p_bytes = 0;              // streaming-equivalent bytes of the batch's FP32 recursions per iteration
+  // cells of the march kernel: their launches go between the batch's two graphs; events around them
+  cudaGraphExec_t bgraph2 = nullptr;
+  cudaEvent_t mev[2] = {nullptr, nullptr};
 
   // autotuned (block_width, cols_per_block, double-step flag, band_rows) per (nx, ny, precision, half pass,
   // probe_p, M)
@@ -186,6 +189,35 @@ void drop_graph(kpm_ctx* ctx) {
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
   ctx->graph = nullptr;
   ctx->key_valid = false;
+}
+
+void drop_batch_graph(kpm_ctx* ctx) {
+  for (cudaGraphExec_t* g : {&ctx->bgraph, &ctx->bgraph2}) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
+  ctx->bkey.clear();
+}
+
+// at least `n` recursion slabs of `bytes` (the first two serve every pass)
+int ensure_slabs(kpm_ctx* ctx, size_t bytes, int n) {
+  if (ctx->slab_bytes >= bytes && ctx->slab_n >= n) return KPM_OK;
+  drop_graph(ctx);
+  for (int k = 0; k < 4; ++k) {
+    if (ctx->slab[k]) cudaFree(ctx->slab[k]);
+    ctx->slab[k] = nullptr;
+  }
+  ctx->slab_bytes = 0;
+  ctx->slab_n = 0;
+  for (int k = 0; k < n; ++k) {
+    if (cudaMalloc(&ctx->slab[k], bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(ctx, KPM_ENOMEM, "cudaMalloc of the recursion slabs failed");
+    }
+  }
+  ctx->slab_bytes = bytes;
+  ctx->slab_n = n;
+  return KPM_OK;
 }
 
 int ensure_site_scratch(kpm_ctx* ctx, int N) {
@@ -291,23 +323,7 @@ int ensure_pass_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, con
   const size_t slab = (size_t)D * pp.cheb.ldv * pp.elem;
   const int nslab = pp.cheb.mk.ns > 1 ? 4 : 2;
   int r;
-  if (ctx->slab_bytes < slab || ctx->slab_n < nslab) {
-    drop_graph(ctx);
-    for (int k = 0; k < 4; ++k) {
-      if (ctx->slab[k]) cudaFree(ctx->slab[k]);
-      ctx->slab[k] = nullptr;
-    }
-    ctx->slab_bytes = 0;
-    ctx->slab_n = 0;
-    for (int k = 0; k < nslab; ++k) {
-      if (cudaMalloc(&ctx->slab[k], slab) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(ctx, KPM_ENOMEM, "cudaMalloc of the recursion slabs failed");
-      }
-    }
-    ctx->slab_bytes = slab;
-    ctx->slab_n = nslab;
-  }
+  if ((r = ensure_slabs(ctx, slab, nslab))) return r;
   const size_t accb = (size_t)D * kSlots * sizeof(double2);
   if (ctx->acc_bytes < accb) drop_graph(ctx);
   if ((r = ensure(ctx, &ctx->acc, &ctx->acc_bytes, accb))) return r;
@@ -342,6 +358,27 @@ int ensure_pass_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, con
   cudaError_t e = cheb_prepare(pp.cheb, o->precision);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cheb_prepare");
   return KPM_OK;
+}
+
+// V_1 .. V_{M-1} of a unit-vector slab by single steps of the march kernel, from V_0 in
+// slab[0], with their moment sums: part of the columns after part (march_columns), each
+// through all its steps.  V_{M-1} ends in slab[(M - 1) & 1].
+cudaError_t enqueue_parts(const ChebPlan& p, const void* table, void* const* slab, int64_t s0, double2* acc,
+                          const double* am, const double* ao, int M, cudaStream_t s, int* launches) {
+  SlabMaps maps[2];
+  for (int k = 0; k < 2; ++k) {
+    const cudaError_t e = encode_slab_maps(p, p.m1, slab[k], &maps[k]);
+    if (e != cudaSuccess) return e;
+  }
+  for (int64_t col = 0; col < p.ldv; col += p.sub)
+    for (int mm = 0; mm < M - 1; ++mm) {
+      // V_{mm+1} in place over V_{mm-1}
+      const cudaError_t e = launch_march(p, p.m1, table, maps[mm & 1], maps[(mm & 1) ^ 1], nullptr, slab[(mm & 1) ^ 1], s0,
+                                         acc, am, ao, mm, mm == 0, s, col, p.sub);
+      if (e != cudaSuccess) return e;
+      *launches += 1;
+    }
+  return cudaSuccess;
 }
 
 // enqueue one KPM pass: fields + ab (device) -> obs, omega
@@ -389,19 +426,12 @@ int enqueue_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, const Pass
     KPM_CU(launch_cheb_init(p, prec, ctx->slab[0], s0, ctx->acc, ctx->am, ctx->ao, s));
     nl += 1;
     if (events && s0 == pp.c0) KPM_CU(cudaEventRecordWithFlags(ctx->ev[0], s, cudaEventRecordExternal));
-    // a single step per launch: part of the columns after part, each through all its steps
-    for (int64_t col = 0; p.mk.ns == 1 && p.sub < p.ldv && col < p.ldv; col += p.sub) {
-      const double part = (double)std::min(p.sub, p.ldv - col) / (double)p.ldv;
-      ix = iy = 0;
-      for (mm = 0; mm < M - 1; ++mm) {
-        const int io = mm == 0 ? 1 : ix;
-        KPM_CU(launch_march(p, p.m1, table1, m1[iy], m1[ix], nullptr, ctx->slab[io], s0, ctx->acc, ctx->am, ctx->ao,
-                            mm, mm == 0, s, col, p.sub));
-        nb += (mm == 0 ? 2 : 3) * vec * part;
-        ix = iy;
-        iy = io;
-        nr += 1;
-      }
+    if (p.mk.ns == 1 && !p.raw && M >= 2) {
+      KPM_CU(enqueue_parts(p, table1, ctx->slab, s0, ctx->acc, ctx->am, ctx->ao, M, s, &nr));
+      nb += (3.0 * (M - 1) - 1.0) * vec;
+      mm = M - 1;
+      iy = mm & 1;
+      ix = iy ^ 1;
     }
     while (mm < M - 1) {
       const bool first = mm == 0;
@@ -586,11 +616,11 @@ int kpm_destroy(kpm_ctx* ctx) {
                   (void*)ctx->dphi, (void*)ctx->misc, ctx->bwd, (void*)ctx->Gacc, (void*)ctx->wseed})
     if (p) cudaFree(p);
   if (ctx->host_misc) cudaFreeHost(ctx->host_misc);
-  if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
+  drop_batch_graph(ctx);
   for (auto& c : ctx->cells)
     if (c.mem) cudaFree(c.mem);
   if (ctx->pbuf) cudaFree(ctx->pbuf);
-  for (cudaEvent_t e : ctx->pev)
+  for (cudaEvent_t e : {ctx->pev[0], ctx->pev[1], ctx->mev[0], ctx->mev[1]})
     if (e) cudaEventDestroy(e);
   for (cudaStream_t st : ctx->fork) cudaStreamDestroy(st);
   for (cudaEvent_t e : ctx->fork_ev) cudaEventDestroy(e);
@@ -1239,26 +1269,31 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   for (size_t k = 0; k < members.size(); ++k) {
     const kpm_model& m0 = models[members[k][0]];
     const int64_t D = 2 * (int64_t)m0.nx * m0.ny;
-    plans[k] = plan_cheb(m0.nx, m0.ny, D, prec, opts->cols_per_block, opts->band_rows, 1);
+    plans[k] = plan_cheb(m0.nx, m0.ny, D, prec, opts->cols_per_block, opts->band_rows, 1, true);
     if (plans[k].cb == 0) return fail(ctx, KPM_EINVAL, "lattice row too wide for the shared-memory window");
     cudaError_t e = cheb_prepare(plans[k], prec);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "prepare");
   }
 
-  // FP32 shape classes whose band of a cell fits shared memory run the
-  // persistent recursion (one launch for all of them, all M moments on chip);
-  // the others keep one batched step launch per moment
+  // Small FP32 cells run the persistent recursion (one launch for all of them, all M
+  // moments on chip), as far as a band of the cell fits shared memory: their launches
+  // would be mostly start.  us per cell and step, persistent against the march kernel:
+  // 12x12 2.6 / 5.5, 16x16 4.3 / 5.8, 24x16 7.0 / 6.2, 24x24 12.8 / 7.8, 32x32 27 / 15.6.
+  // The others run the march kernel one after the other, over one pair of slabs, unless
+  // the slabs do not fit the budget or the device; their launches go between two graphs
+  // (a graph of them has cells x parts x M nodes).
+  constexpr int64_t kPersistRows = 640;
   std::vector<char> persist(members.size(), 0);
-  size_t psmem = 0;
+  size_t psmem = 0, march_slab = 0;
   int pclusters = 0;
-  if (prec == KPM_FP32 && M >= 1) {
+  for (int small = 1; prec == KPM_FP32 && small >= 0; --small) {
+    psmem = march_slab = 0;
     for (size_t k = 0; k < members.size(); ++k) {
       const kpm_model& m0 = models[members[k][0]];
       const size_t sm = persist_smem_bytes(m0.nx, m0.ny);
-      if (sm <= 227 * 1024) {
-        persist[k] = 1;
-        psmem = std::max(psmem, sm);
-      }
+      const size_t slab = (size_t)plans[k].D * plans[k].ldv * elem;
+      persist[k] = sm <= 227 * 1024 && (!small || plans[k].D <= kPersistRows || 2 * slab > ctx->budget);
+      if (persist[k]) psmem = std::max(psmem, sm);
     }
     if (psmem > 0) {
       cudaError_t e = persist_prepare(psmem, &pclusters);
@@ -1268,7 +1303,17 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
         psmem = 0;
       }
     }
+    for (size_t k = 0; k < members.size(); ++k)
+      if (!persist[k]) march_slab = std::max(march_slab, (size_t)plans[k].D * plans[k].ldv * elem);
+    r = march_slab > 0 ? ensure_slabs(ctx, march_slab, 2) : KPM_OK;
+    if (r == KPM_OK) break;
+    if (!small) return r;
   }
+  for (int k = 0; k < 2 && march_slab > 0; ++k)
+    if (!ctx->mev[k] && cudaEventCreate(&ctx->mev[k]) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(ctx, KPM_ECUDA, "event creation failed");
+    }
 
   // per-cell scratch, one allocation per cell
   auto al = [](size_t n) { return (n + 255) & ~(size_t)255; };
@@ -1281,15 +1326,13 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     const int N = models[c].nx * models[c].ny;
     const int64_t D = 2 * (int64_t)N;
     const int k = cls_of[std::make_pair(models[c].nx, models[c].ny)];
-    // (cells of the persistent recursion keep their vectors in shared memory: no slabs)
+    // (FP32 cells keep their vectors in shared memory or share the pass's slabs)
     need[c] = al(26 * (size_t)N * 8) * 2 + al((size_t)M * 8) * 2 + al(16 * 8) + al((size_t)D * kSlots * 16) +
-              al(tab_bytes(k, N)) + (persist[k] ? 0 : 2 * al((size_t)D * plans[k].ldv * elem));
+              al(tab_bytes(k, N)) + (prec == KPM_FP32 ? 0 : 2 * al((size_t)D * plans[k].ldv * elem));
     if (!realloc && ctx->cells[c].bytes < need[c]) realloc = true;
   }
   if (realloc) {
-    if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
-    ctx->bgraph = nullptr;
-    ctx->bkey.clear();
+    drop_batch_graph(ctx);
     for (auto& c : ctx->cells)
       if (c.mem) cudaFree(c.mem);
     ctx->cells.assign(ncell, kpm_ctx::Cell());
@@ -1315,7 +1358,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     C.misc = (double*)b; b += al(16 * 8);
     C.acc = (double2*)b; b += al((size_t)D * kSlots * 16);
     C.table = b; b += al(tab_bytes(k, N));
-    if (persist[k]) {
+    if (prec == KPM_FP32) {
       C.A = C.B = nullptr;
     } else {
       C.A = b; b += al((size_t)D * plans[k].ldv * elem);
@@ -1335,9 +1378,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
       return fail(ctx, KPM_ENOMEM, "cudaMallocHost failed");
     }
     ctx->bhost_n = (size_t)ncell * 16;
-    if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
-    ctx->bgraph = nullptr;
-    ctx->bkey.clear();
+    drop_batch_graph(ctx);
   }
   while (ctx->fork.size() < members.size()) {
     cudaStream_t st;
@@ -1365,9 +1406,9 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   put(phis, sizeof(double*) * ncell);
   put(params, sizeof(double*) * ncell);
   put(&mu_eff, sizeof(mu_eff));
+  put(persist.data(), persist.size());
   if (!ctx->bgraph || key != ctx->bkey) {
-    if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
-    ctx->bgraph = nullptr;
+    drop_batch_graph(ctx);
     cudaStream_t c0 = ctx->cap;
     // persistent recursion: the cell table and the work items, longest first
     // (an item's time grows with its cell's band, nx ceil(ny / kPClu) sites),
@@ -1389,7 +1430,6 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
         const int64_t D = 2 * (int64_t)models[c].nx * models[c].ny;
         nx_max = std::max(nx_max, models[c].nx);
         for (int64_t q0 = 0; q0 < D; q0 += q) hi.push_back(PItem{c, (int)q0});
-        pbytes += 24.0 * (double)D * (double)D * (double)std::max(0, M - 1);
       }
       std::stable_sort(hi.begin(), hi.end(), [&](const PItem& a, const PItem& b) {
         auto cost = [&](const PItem& t) {
@@ -1417,6 +1457,10 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
           return fail(ctx, KPM_ECUDA, "event creation failed");
         }
     }
+    for (int c = 0; c < ncell && prec == KPM_FP32; ++c) {
+      const double D = 2.0 * models[c].nx * models[c].ny;
+      pbytes += 24.0 * D * D * (double)std::max(0, M - 1);
+    }
     ctx->p_bytes = pbytes;
     ctx->p_launched = nitems > 0;
 
@@ -1443,12 +1487,12 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
         KPM_TRY(launch_scale_table_f32(m, C.fields, C.misc, (float2*)C.table, c0));
       else
         KPM_TRY(launch_march_table(m, p.m1, C.fields, C.misc, (float4*)C.table, c0));
-      if (!persist[C.cls]) KPM_TRY(launch_cheb_init(p, prec, C.A, 0, C.acc, C.am, C.ao, c0));
+      if (prec != KPM_FP32) KPM_TRY(launch_cheb_init(p, prec, C.A, 0, C.acc, C.am, C.ao, c0));
     }
-    // recursion: one chain per shape class on its own stream
+    // FP64 recursion: one chain per shape class on its own stream
     KPM_TRY(cudaEventRecord(ctx->join_ev, c0));
     for (size_t k = 0; k < members.size() && M >= 2; ++k) {
-      if (persist[k]) continue;
+      if (prec == KPM_FP32) break;
       cudaStream_t sk = ctx->fork[k];
       KPM_TRY(cudaStreamWaitEvent(sk, ctx->join_ev, 0));
       const ChebPlan& p = plans[k];
@@ -1465,18 +1509,25 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
       KPM_TRY(cudaStreamWaitEvent(c0, ctx->fork_ev[k], 0));
     }
     if (nitems > 0) {
-      // every moment of every persistent cell in one launch, concurrent with
-      // the per-step launches of the other shape classes
+      // every moment of every persistent cell in one launch
       KPM_TRY(cudaMemsetAsync(d_counter, 0, sizeof(int), c0));
       KPM_TRY(cudaEventRecordWithFlags(ctx->pev[0], c0, cudaEventRecordExternal));
       KPM_TRY(launch_cheb_persist(d_cells, d_items, nitems, d_counter, M, nclu, psmem, d_xbuf, nx_max, c0));
       KPM_TRY(cudaEventRecordWithFlags(ctx->pev[1], c0, cudaEventRecordExternal));
     }
+    if (march_slab > 0) {
+      // the march cells' recursions are launched here; then the second graph
+      cudaGraph_t first = nullptr;
+      KPM_TRY(cudaStreamEndCapture(c0, &first));
+      KPM_TRY(cudaGraphInstantiate(&ctx->bgraph, first, 0));
+      if (first) cudaGraphDestroy(first);
+      KPM_TRY(cudaStreamBeginCapture(c0, cudaStreamCaptureModeThreadLocal));
+    }
     for (int c = 0; c < ncell; ++c) {
       kpm_ctx::Cell& C = ctx->cells[c];
       const int N = models[c].nx * models[c].ny;
       const ChebPlan& p = plans[C.cls];
-      if (M >= 2 && !persist[C.cls])
+      if (M >= 2 && prec != KPM_FP32)
         KPM_TRY(launch_cheb_gather(p, prec, ((M - 1) & 1) ? C.B : C.A, 0, C.acc, C.am, C.ao, M - 1, c0));
       KPM_TRY(launch_assemble(models[c].nx, models[c].ny, C.acc, C.misc, C.obs, C.misc + 3, ctx->bred, c0));
       KPM_TRY(launch_update(N, params[c], C.obs, mu_eff + c, ropts[c], C.misc + 4, ctx->bred, c0));
@@ -1487,13 +1538,17 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     cudaError_t e2 = cudaStreamEndCapture(c0, &graph);
     if (e != cudaSuccess) {
       if (graph) cudaGraphDestroy(graph);
+      drop_batch_graph(ctx);
       return cuda_fail(ctx, e, (std::string("capture of the batched iteration at ") + where).c_str());
     }
-    if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(&ctx->bgraph, graph, 0);
+    if (e2 != cudaSuccess) {
+      drop_batch_graph(ctx);
+      return cuda_fail(ctx, e2, "cudaStreamEndCapture");
+    }
+    e = cudaGraphInstantiate(march_slab > 0 ? &ctx->bgraph2 : &ctx->bgraph, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
-      ctx->bgraph = nullptr;
+      drop_batch_graph(ctx);
       return cuda_fail(ctx, e, "cudaGraphInstantiate");
     }
     ctx->bkey = key;
@@ -1504,9 +1559,30 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   memset(st.data(), 0, sizeof(kpm_rmft_stats) * ncell);
   int status = KPM_OK;
   double pms = 0.0;
+  int rec_launches = ctx->p_launched;
   for (int it = 0; it < n_iter; ++it) {
     KPM_CU(cudaGraphLaunch(ctx->bgraph, s));
+    if (march_slab > 0) {
+      int launched = ctx->p_launched;
+      KPM_CU(cudaEventRecord(ctx->mev[0], s));
+      for (int c = 0; c < ncell; ++c) {
+        const kpm_ctx::Cell& C = ctx->cells[c];
+        if (persist[C.cls]) continue;
+        const ChebPlan& p = plans[C.cls];
+        KPM_CU(launch_cheb_init(p, prec, ctx->slab[0], 0, C.acc, C.am, C.ao, s));
+        KPM_CU(enqueue_parts(p, C.table, ctx->slab, 0, C.acc, C.am, C.ao, M, s, &launched));
+        if (M >= 2) KPM_CU(launch_cheb_gather(p, prec, ctx->slab[(M - 1) & 1], 0, C.acc, C.am, C.ao, M - 1, s));
+      }
+      KPM_CU(cudaEventRecord(ctx->mev[1], s));
+      rec_launches = launched;
+      KPM_CU(cudaGraphLaunch(ctx->bgraph2, s));
+    }
     KPM_CU(cudaStreamSynchronize(s));
+    if (march_slab > 0) {
+      float ms = 0.f;
+      KPM_CU(cudaEventElapsedTime(&ms, ctx->mev[0], ctx->mev[1]));
+      pms += ms;
+    }
     if (ctx->p_launched) {
       float ms = 0.f;
       KPM_CU(cudaEventElapsedTime(&ms, ctx->pev[0], ctx->pev[1]));
@@ -1532,12 +1608,12 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     }
     if (status != KPM_OK || all) break;
   }
-  // the persistent launch serves every cell: its time and streaming-equivalent
-  // bytes are reported on each cell of the batch
+  // the FP32 recursions' time, streaming-equivalent bytes and launches (of an
+  // iteration) are the batch's, reported on each cell
   for (auto& q : st) {
     q.recursion_ms = pms;
-    q.recursion_bytes = ctx->p_launched ? ctx->p_bytes * (double)(q.iterations) : 0.0;
-    q.recursion_launches = ctx->p_launched ? 1 : 0;
+    q.recursion_bytes = ctx->p_bytes * (double)(q.iterations);
+    q.recursion_launches = rec_launches;
   }
   if (stats) memcpy(stats, st.data(), sizeof(kpm_rmft_stats) * ncell);
   return status;
