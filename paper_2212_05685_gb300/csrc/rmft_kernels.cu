@@ -71,6 +71,7 @@ struct SiteF {
   double gxy, dgxy[2];
 };
 
+template <bool DERIV = true>  // with the derivatives (else dgt and dgxy are not set)
 __device__ SiteF site_factors(double nu, double nd, bool gutz) {
   SiteF f;
   f.delta = 1.0 - nu - nd;
@@ -92,14 +93,16 @@ __device__ SiteF site_factors(double nu, double nd, bool gutz) {
     const double up = 1.0 + de + 2.0 * sg * m;
     const double dn = 1.0 + de - 2.0 * sg * m;
     const double g = sqrt(2.0 * de * (1.0 - de) / Pe * up / dn);
+    f.gt[s] = g;
+    if (!DERIV) continue;
     double dld = 1.0 / de - 1.0 / (1.0 - de) + 2.0 * de / Pe + 1.0 / up - 1.0 / dn;
     if (clamped) dld = 0.0;
     const double dlm = -8.0 * m / Pe + 2.0 * sg / up + 2.0 * sg / dn;
-    f.gt[s] = g;
     f.dgt[s][0] = 0.5 * g * (-dld + 0.5 * dlm);
     f.dgt[s][1] = 0.5 * g * (-dld - 0.5 * dlm);
   }
   f.gxy = 2.0 * (1.0 - f.delta) / f.P;
+  if (!DERIV) return f;
   const double ld = -1.0 / (1.0 - f.delta) + 2.0 * f.delta / f.P;
   const double lm = -8.0 * m / f.P;
   f.dgxy[0] = f.gxy * (-ld + 0.5 * lm);
@@ -347,26 +350,29 @@ __global__ void shift_eps_kernel(int N, double* __restrict__ fld, const double* 
   if (blockIdx.x == 0 && threadIdx.x == 0 && mu_out) *mu_out = *mu_eff + mean;
 }
 
-// Gershgorin row bounds: per site the max of h_II + R_I and min of h_II - R_I
+// Gershgorin row bounds: the max of h_II + R_I and min of h_II - R_I.  FP64 work (twelve
+// moduli a row) bounds it: a thread per Nambu row and blocks of kGershBlock, so that all
+// SMs have some (a thread per site in blocks of 256, 40 of them at 100x100: 35.0 ->
+// 19.1 us).  The rows' sums and the extrema do not depend on the split.
+constexpr int kGershBlock = 128;
 __global__ void gershgorin_partial(kpm_model m, const double* __restrict__ fld, double* __restrict__ part) {
   const int nx = m.nx, ny = m.ny, N = nx * ny;
   const Layout L{N};
   double hi = -INFINITY, lo = INFINITY;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    double R0 = 0.0, R1 = 0.0;
+  for (int I = blockIdx.x * blockDim.x + threadIdx.x; I < 2 * N; I += gridDim.x * blockDim.x) {
+    const int r = I >= N, i = I - r * N;
+    double R = 0.0;
     for (int d = 0; d < 4; ++d) {
       const int k = shift(i, -kFwdX[d], -kFwdY[d], nx, ny);
-      R0 += cabs(L.chi(fld, 0, d, i)) + cabs(L.chi(fld, 0, d, k));
-      R1 += cabs(L.chi(fld, 1, d, i)) + cabs(L.chi(fld, 1, d, k));
+      R += cabs(L.chi(fld, r, d, i)) + cabs(L.chi(fld, r, d, k));
     }
     for (int e = 0; e < 4; ++e) {
       const int j = shift(i, kNnX[e], kNnY[e], nx, ny);
-      R0 += cabs(L.F(fld, e, i));
-      R1 += cabs(L.F(fld, (e + 2) & 3, j));
+      R += r ? cabs(L.F(fld, (e + 2) & 3, j)) : cabs(L.F(fld, e, i));
     }
-    const double d0 = L.n(fld, 0, i), d1 = -L.n(fld, 1, i);
-    hi = fmax(hi, fmax(d0 + R0, d1 + R1));
-    lo = fmin(lo, fmin(d0 - R0, d1 - R1));
+    const double d0 = r ? -L.n(fld, 1, i) : L.n(fld, 0, i);
+    hi = fmax(hi, d0 + R);
+    lo = fmin(lo, d0 - R);
   }
   hi = block_reduce<1>(hi);
   lo = block_reduce<2>(lo);
@@ -925,7 +931,9 @@ cudaError_t launch_peierls(const kpm_model& m, double* phi, cudaStream_t s) {
 cudaError_t launch_fields(const kpm_model& m, const double* phi, const double* params, double mu,
                           double* fields, double* wsite, cudaStream_t s) {
   const int N = m.nx * m.ny;
-  fields_kernel<<<(N + 127) / 128, 128, 0, s>>>(m, phi, params, mu, fields, wsite);
+  // a warp per block: FP64 work bounds the kernel, and 313 of them (100x100) are spread more
+  // evenly over the SMs than 79 blocks of four: 74.8 -> 74.0 us
+  fields_kernel<<<(N + 31) / 32, 32, 0, s>>>(m, phi, params, mu, fields, wsite);
   return cudaGetLastError();
 }
 
@@ -947,8 +955,8 @@ cudaError_t launch_shift_eps(int N, double* fields, const double* mu_eff, double
 cudaError_t launch_gershgorin(const kpm_model& m, const double* fields, double margin, double* ab, double* red,
                               cudaStream_t s, int symmetric) {
   const int N = m.nx * m.ny;
-  const int g = grid_for(N);
-  gershgorin_partial<<<g, kRedBlock, 0, s>>>(m, fields, red);
+  const int g = std::min((2 * N + kGershBlock - 1) / kGershBlock, kRedGrid);
+  gershgorin_partial<<<g, kGershBlock, 0, s>>>(m, fields, red);
   gershgorin_final<<<1, kRedBlock, 0, s>>>(red, g, margin, symmetric, ab);
   return cudaGetLastError();
 }
@@ -1014,44 +1022,64 @@ __global__ void coefficients_T_kernel(int M, const double* __restrict__ ab, doub
 // Delta_{i,i+tau,sigma} e^{i phi_{i,i+tau}} (Delta_up = F_ij, Delta_dn = F_ji; the
 // bond phase sign makes Delta_i a pair at site i under gauge changes) and
 // M_i = (-1)^{x+y} g^xy_i/4 sum_tau sqrt(R_{i,i+tau}) m_i (R = g^z/g^xy).
-__global__ void order_parameters_kernel(kpm_model m, const double* __restrict__ phi, const double* __restrict__ p,
-                                        double* __restrict__ delta_out, double* __restrict__ mag_out) {
+// FP64 work bounds the kernel.  Tiles of kTW x kTH sites, a warp: the Gutzwiller factors of
+// a tile's sites and of those around are computed once (60 for 32 sites; one thread per
+// site computed 5 of them a site, on the few warps that 10^4 sites make) into shared
+// memory, then a warp takes each nearest neighbour.  100x100: 30.5 -> 14.5 us.
+constexpr int kTW = 8, kTH = 4, kTileHalo = (kTW + 2) * (kTH + 2);
+int tile_grid(const kpm_model& m) { return ((m.nx + kTW - 1) / kTW) * ((m.ny + kTH - 1) / kTH); }
+__global__ void __launch_bounds__(128)
+    order_parameters_kernel(kpm_model m, const double* __restrict__ phi, const double* __restrict__ p,
+                            double* __restrict__ delta_out, double* __restrict__ mag_out) {
+  __shared__ SiteF sf[kTileHalo];
+  __shared__ Cplx d_part[4][32];
+  __shared__ double r_part[4][32];
   const int nx = m.nx, ny = m.ny, N = nx * ny;
   const Layout L{N};
   const bool gutz = m.gutzwiller != 0;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const SiteF si = site_factors(L.n(p, 0, i), L.n(p, 1, i), gutz);
-  Cplx dsum = cx(0.0, 0.0);
-  double rsum = 0.0;
-  for (int e = 0; e < 4; ++e) {
+  const int e = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tiles = (nx + kTW - 1) / kTW, x0 = blockIdx.x % tiles * kTW, y0 = blockIdx.x / tiles * kTH;
+  if (threadIdx.x < kTileHalo) {
+    const int j = site_of(x0 - 1 + (int)threadIdx.x % (kTW + 2), y0 - 1 + (int)threadIdx.x / (kTW + 2), nx, ny);
+    sf[threadIdx.x] = site_factors<false>(L.n(p, 0, j), L.n(p, 1, j), gutz);
+  }
+  __syncthreads();
+  const int x = x0 + lane % kTW, y = y0 + lane / kTW, at = (lane / kTW + 1) * (kTW + 2) + lane % kTW + 1;
+  const bool in = x < nx && y < ny;
+  const int i = in ? x + nx * y : 0;
+  const SiteF& si = sf[at];
+  if (in) {
     const int j = shift(i, kNnX[e], kNnY[e], nx, ny);
-    const SiteF sj = site_factors(L.n(p, 0, j), L.n(p, 1, j), gutz);
+    const SiteF& sj = sf[at + kNnY[e] * (kTW + 2) + kNnX[e]];
     // phase of the bond i -> j: forward +x/+y stored at i, -x/-y minus the forward phase at j
     const double ph = e < 2 ? phi[e * N + i] : -phi[(e - 2) * N + j];
     double sn, cs;
     sincos(ph, &sn, &cs);
     const Cplx term = cadd(cscale(L.F(p, e, i), si.gt[0] * sj.gt[0]), cscale(L.F(p, (e + 2) & 3, j), si.gt[1] * sj.gt[1]));
-    dsum = cadd(dsum, cscale(cmul(term, cx(cs, sn)), e == 1 || e == 3 ? -1.0 : 1.0));
+    d_part[e][lane] = cscale(cmul(term, cx(cs, sn)), e == 1 || e == 3 ? -1.0 : 1.0);
     // exchange ratio R of the bond (stored at its forward end)
     const int d = e & 1;
     const int a = e < 2 ? i : j, b = e < 2 ? j : i;
-    const SiteF& sa = e < 2 ? si : sj;
-    const SiteF& sb = e < 2 ? sj : si;
-    const BondX bx = bond_exchange(sa, sb, L.chi(p, 0, d, a), L.chi(p, 1, d, a), L.F(p, d, a), L.F(p, d + 2, b),
-                                   m.J, gutz);
-    rsum += sqrt(bx.R);
+    const BondX bx = bond_exchange(e < 2 ? si : sj, e < 2 ? sj : si, L.chi(p, 0, d, a), L.chi(p, 1, d, a), L.F(p, d, a),
+                                   L.F(p, d + 2, b), m.J, gutz);
+    r_part[e][lane] = sqrt(bx.R);
+  }
+  __syncthreads();
+  if (!in || e != 0) return;
+  Cplx dsum = cx(0.0, 0.0);
+  double rsum = 0.0;
+  for (int k = 0; k < 4; ++k) {
+    dsum = cadd(dsum, d_part[k][lane]);
+    rsum += r_part[k][lane];
   }
   delta_out[2 * i] = dsum.re / 8.0;
   delta_out[2 * i + 1] = dsum.im / 8.0;
-  const int x = i % nx, y = i / nx;
   mag_out[i] = ((x + y) & 1 ? -1.0 : 1.0) * si.gxy / 4.0 * rsum * si.m;
 }
 
 cudaError_t launch_order_parameters(const kpm_model& m, const double* phi, const double* params, double* delta_out,
                                     double* mag_out, cudaStream_t s) {
-  const int N = m.nx * m.ny;
-  order_parameters_kernel<<<(N + 127) / 128, 128, 0, s>>>(m, phi, params, delta_out, mag_out);
+  order_parameters_kernel<<<tile_grid(m), 128, 0, s>>>(m, phi, params, delta_out, mag_out);
   return cudaGetLastError();
 }
 
