@@ -931,9 +931,7 @@ cudaError_t launch_peierls(const kpm_model& m, double* phi, cudaStream_t s) {
 cudaError_t launch_fields(const kpm_model& m, const double* phi, const double* params, double mu,
                           double* fields, double* wsite, cudaStream_t s) {
   const int N = m.nx * m.ny;
-  // a warp per block: FP64 work bounds the kernel, and 313 of them (100x100) are spread more
-  // evenly over the SMs than 79 blocks of four: 74.8 -> 74.0 us
-  fields_kernel<<<(N + 31) / 32, 32, 0, s>>>(m, phi, params, mu, fields, wsite);
+  fields_kernel<<<(N + 127) / 128, 128, 0, s>>>(m, phi, params, mu, fields, wsite);
   return cudaGetLastError();
 }
 
