@@ -398,9 +398,7 @@ def run_ours(args):
     alg_bytes = rec_bytes / max(rec_launches, 1)
     vecs_per_launch = alg_bytes / (D * ldv * 8)
     dbl = vecs_per_launch > 3.5
-    # single step: chunks of 8 or 16 columns run the TMA-staged kernel
-    kname = "cheb_step2_f32_kernel" if dbl else (
-        "cheb_step_f32_tma_kernel<%d,1>" % cb if cb >= 8 else "cheb_step_f32_kernel<%d,1>" % cb)
+    kname = "cheb_march_kernel, several steps per launch" if dbl else "cheb_march_kernel, one step per launch"
     pk, pk_kind = peaks()
     achieved = rec_bytes / (rec_ms / 1e3) / 1e9
     nslab = 4 if dbl else 2
@@ -596,10 +594,9 @@ def run_ours(args):
 
 def batched_section(kpm, inputs, torch, alu=None, iters=3):
     """32 cells of uneven size and doping (shapes 24x12 .. 64x32), M = 1024,
-    FP32: one batched graph per iteration (the persistent recursion: every
-    moment of every cell in one launch, vectors on chip) vs the cells one
-    after another; roofline of the persistent launch against the measured FP32
-    FMA rate (its vectors never leave shared memory)."""
+    FP32: the batched call (cells of up to 640 Nambu rows in one persistent launch,
+    the others on the march kernel) vs the cells one after another; roofline of
+    the batch's recursions against the measured FP32 FMA rate."""
     cells = inputs.cfg3_cells(seed=0, count=32)
     M = 1024
     opts = kpm.make_opts(M, kpm.KPM_FP32)
@@ -647,7 +644,7 @@ def batched_section(kpm, inputs, torch, alu=None, iters=3):
             "s_per_iteration": rec_s, "launches_per_iteration": bst[0].recursion_launches,
             "effective_gbs": 24.0 * row_updates / rec_s / 1e9,
             "effective_note": "24 B per row-column (read V_m, V_m-1, write V_m+1) as if streamed; the vectors stay "
-                              "in shared memory",
+                              "in shared memory (small cells) or mostly in L2",
             "roofline": {"bound": "alu", "achieved": tflops, "peak": alu[1] if alu else None, "unit": "TFLOP/s",
                          "frac": tflops / alu[1] if alu else None,
                          "peak_kind": "measured FP32 FMA rate (kpm_measure_peaks)"}}
@@ -1062,7 +1059,7 @@ def profile_probing():
 
 def profile_batched():
     """Small batch for ncu: 4 cells of 48x24 and 2 of 64x32, M = 64, FP32,
-    one iteration of the batched call (one persistent recursion launch)."""
+    one iteration of the batched call (march kernel launches)."""
     import torch
     from paper_2212_05685_gb300 import build, inputs, kpm
     build.build()

@@ -201,7 +201,7 @@ int kpm_set_scratch_budget(kpm_ctx* ctx, uint64_t bytes);
  * word themselves when an iteration turns non-finite. */
 int kpm_sync_status(kpm_ctx* ctx, void* stream);
 /* Failure-path test hook (no counterpart in the paper).  The next `count` CTAs
- * of the TMA-staged FP32 recursion step that would issue the copy of their
+ * of the recursion's march kernel that would issue the copy of their
  * third window row skip that copy and its expected byte count, so nothing is
  * in flight for that slot and the CTA's bounded waits expire: the launch
  * writes NaN and the fault word reads KPM_ETIMEDOUT, with no device fault.
@@ -293,7 +293,7 @@ int rmft_update(kpm_ctx* ctx, const kpm_model* model, const kpm_rmft_opts* ropts
 /* Autotuner of the recursion launch: times two short passes (M = 18 and 34)
  * for every slab width in {D, 8192, ..., 128} (narrow slabs keep both
  * recursion vectors in L2), every column chunk that fits shared memory and
- * (FP32) one or two steps per launch, and for one step per launch the
+ * (FP32) the default steps per launch or one more, and for the default the
  * three best band heights of a wave model of the launch (CTAs of
  * ceil(ny / bands) rows, one per SM; the first is the default of band_rows
  * = 0) and one band per column chunk, predicts the pass at opts->M from the
