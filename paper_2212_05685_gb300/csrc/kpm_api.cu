@@ -108,6 +108,8 @@ struct kpm_ctx {
   double p_bytes = 0;              // streaming-equivalent bytes of the batch's FP32 recursions per iteration
   // cells of the march kernel: their launches go between the batch's two graphs; events around them
   cudaGraphExec_t bgraph2 = nullptr;
+  void* bslab[2] = {nullptr, nullptr};  // their slabs (not the passes': those may run on another stream)
+  size_t bslab_bytes[2] = {0, 0};
   cudaEvent_t mev[2] = {nullptr, nullptr};
 
   // autotuned (block_width, cols_per_block, double-step flag, band_rows) per (nx, ny, precision, half pass,
@@ -610,7 +612,7 @@ int kpm_destroy(kpm_ctx* ctx) {
   drop_graph(ctx);
   cublas_destroy(ctx->cublas);
   for (void* p : {ctx->slab[0], ctx->slab[1], ctx->slab[2], ctx->slab[3], (void*)ctx->xi, (void*)ctx->ldos_buf,
-                  (void*)ctx->and_buf, (void*)ctx->peak_buf, ctx->tail, (void*)ctx->tail_in,
+                  (void*)ctx->and_buf, (void*)ctx->peak_buf, ctx->bslab[0], ctx->bslab[1], ctx->tail, (void*)ctx->tail_in,
                   (void*)ctx->acc, ctx->table, (void*)ctx->am, (void*)ctx->ao,
                   (void*)ctx->red, (void*)ctx->fields, (void*)ctx->obs, (void*)ctx->wsite, (void*)ctx->dparams,
                   (void*)ctx->dphi, (void*)ctx->misc, ctx->bwd, (void*)ctx->Gacc, (void*)ctx->wseed})
@@ -1251,7 +1253,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   const int M = opts->M, prec = opts->precision;
   const size_t elem = prec == KPM_FP32 ? 8 : 16;
 
-  // shape classes (cells of equal nx, ny share one batched launch per step)
+  // shape classes (cells of equal nx, ny share a plan)
   std::map<std::pair<int, int>, int> cls_of;
   std::vector<std::vector<int>> members;
   for (int c = 0; c < ncell; ++c) {
@@ -1305,7 +1307,9 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     }
     for (size_t k = 0; k < members.size(); ++k)
       if (!persist[k]) march_slab = std::max(march_slab, (size_t)plans[k].D * plans[k].ldv * elem);
-    r = march_slab > 0 ? ensure_slabs(ctx, march_slab, 2) : KPM_OK;
+    r = KPM_OK;
+    for (int k = 0; k < 2 && r == KPM_OK && march_slab > 0; ++k)
+      r = ensure(ctx, &ctx->bslab[k], &ctx->bslab_bytes[k], march_slab);
     if (r == KPM_OK) break;
     if (!small) return r;
   }
@@ -1326,7 +1330,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     const int N = models[c].nx * models[c].ny;
     const int64_t D = 2 * (int64_t)N;
     const int k = cls_of[std::make_pair(models[c].nx, models[c].ny)];
-    // (FP32 cells keep their vectors in shared memory or share the pass's slabs)
+    // (FP32 cells keep their vectors in shared memory or share one pair of slabs)
     need[c] = al(26 * (size_t)N * 8) * 2 + al((size_t)M * 8) * 2 + al(16 * 8) + al((size_t)D * kSlots * 16) +
               al(tab_bytes(k, N)) + (prec == KPM_FP32 ? 0 : 2 * al((size_t)D * plans[k].ldv * elem));
     if (!realloc && ctx->cells[c].bytes < need[c]) realloc = true;
@@ -1569,9 +1573,9 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
         const kpm_ctx::Cell& C = ctx->cells[c];
         if (persist[C.cls]) continue;
         const ChebPlan& p = plans[C.cls];
-        KPM_CU(launch_cheb_init(p, prec, ctx->slab[0], 0, C.acc, C.am, C.ao, s));
-        KPM_CU(enqueue_parts(p, C.table, ctx->slab, 0, C.acc, C.am, C.ao, M, s, &launched));
-        if (M >= 2) KPM_CU(launch_cheb_gather(p, prec, ctx->slab[(M - 1) & 1], 0, C.acc, C.am, C.ao, M - 1, s));
+        KPM_CU(launch_cheb_init(p, prec, ctx->bslab[0], 0, C.acc, C.am, C.ao, s));
+        KPM_CU(enqueue_parts(p, C.table, ctx->bslab, 0, C.acc, C.am, C.ao, M, s, &launched));
+        if (M >= 2) KPM_CU(launch_cheb_gather(p, prec, ctx->bslab[(M - 1) & 1], 0, C.acc, C.am, C.ao, M - 1, s));
       }
       KPM_CU(cudaEventRecord(ctx->mev[1], s));
       rec_launches = launched;
