@@ -32,7 +32,7 @@
 //
 // Measured against the one-step kernel with block-shared windows, us per step:
 // 37x29 40.0 -> 20.8 (18.3 where launches overlap), 48x24 31.8 -> 16.7 (one step, slabs in L2), 64x64 343 ->
-// 266 (one step, 90% of the copy rate), 100x100 1655 -> 1248 (two steps; one
+// 266 (one step, 90% of the copy rate; 217 in parts that fit L2), 100x100 1655 -> 1248 (two steps; one
 // step: 1457 = 97% of the copy rate), its eighth (2500 columns) 237 -> 180.
 // FP64 and double-float elements (one complex number of 16 bytes in place of a column
 // pair, 24 cmac and two real products a site) are bound by their arithmetic; the march
