@@ -49,7 +49,7 @@ extern "C" {
 #define KPM_ENOMEM (-2)      /* scratch allocation failed */
 #define KPM_ECUDA (-3)       /* a CUDA call failed; kpm_last_error() has the CUDA message */
 #define KPM_ENONFINITE (-4)  /* NaN or Inf in an output */
-#define KPM_ETIMEDOUT (-5)   /* a bounded device wait of the FP32 recursion expired (kpm_sync_status, rmft_iterate) */
+#define KPM_ETIMEDOUT (-5)   /* a bounded device wait of the recursion expired (kpm_sync_status, rmft_iterate) */
 #define KPM_ENOTCONV (-6)    /* rmft_iterate reached n_iter without meeting tol (only if asked to report it) */
 
 #define KPM_FP64 0
@@ -190,9 +190,10 @@ int kpm_destroy(kpm_ctx* ctx);
 /* Upper bound (bytes) on recursion-slab scratch; default 24 GiB. */
 int kpm_set_scratch_budget(kpm_ctx* ctx, uint64_t bytes);
 /* Synchronise `stream` (NULL: the legacy default stream) and read the device
- * fault word of the FP32 recursion: KPM_OK; KPM_ETIMEDOUT when one of its
- * bounded waits for its own TMA copies expired (that launch, and every FP32
- * recursion launch of the process after it until the word is cleared, wrote
+ * fault word of the TMA-staged recursion (FP32, and FP64 and double-float on unit
+ * vectors): KPM_OK; KPM_ETIMEDOUT when one of its
+ * bounded waits for its own TMA copies expired (that launch, and every such
+ * launch of the process after it until the word is cleared, wrote
  * NaN instead of results); KPM_ECUDA for an asynchronous CUDA error or a
  * recursion that found its shared memory misaligned for TMA (outputs NaN as
  * well).  A word that is reported is cleared (after the device is idle), so
@@ -205,8 +206,8 @@ int kpm_sync_status(kpm_ctx* ctx, void* stream);
  * third window row skip that copy and its expected byte count, so nothing is
  * in flight for that slot and the CTA's bounded waits expire: the launch
  * writes NaN and the fault word reads KPM_ETIMEDOUT, with no device fault.
- * wait_limit_s > 0 sets the bounded-wait limit of every later FP32 recursion
- * launch in the process (default 2 s); <= 0 restores the default.  count = 0
+ * wait_limit_s > 0 sets the bounded-wait limit of every later TMA-staged
+ * recursion launch in the process (default 2 s); <= 0 restores the default.  count = 0
  * withdraws outstanding skips.  Synchronises the device. */
 int kpm_inject_lost_copy(kpm_ctx* ctx, int count, double wait_limit_s);
 /* Measured ALU peaks of the device (no counterpart in the paper; the
@@ -250,10 +251,11 @@ int kpm_bounds(kpm_ctx* ctx, const kpm_model* model, const double* fields,
  * energy 0; omega = a tr G_M(h~) with G_M the damped series of min(x - x0, 0).
  * fields, ab: device (ab as written by kpm_bounds).  obs: device 26*N,
  * written.  omega: device double or NULL.
- * Asynchronous on `stream`.  The FP32 recursion moves its rows by TMA copies
+ * Asynchronous on `stream`.  The recursion (FP64 and double-float: on unit
+ * vectors) moves its rows by TMA copies
  * that complete on mbarriers; its waits are bounded in time (2 s), and a
  * recursion whose copies never land writes NaN over the rows it owns (and
- * every later FP32 recursion launch of the process does the same), so such a
+ * every later launch of the kind in the process does the same), so such a
  * device failure shows as NaN in obs and as KPM_ETIMEDOUT from
  * kpm_sync_status and rmft_iterate, rather than as a hang. */
 int kpm_observables(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts,
@@ -381,7 +383,7 @@ int kpm_backward(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
  * Arguments as for kpm_observables (all sites: site_begin = site_end = 0;
  * negative block_width or cols_per_block: KPM_EINVAL), device pointers of the
  * current device; result within rounding of kpm_observables (identical
- * arithmetic, possibly a different slab width).  The FP32 recursion's bounded
+ * arithmetic, possibly a different slab width).  The recursion's bounded
  * waits behave as in kpm_observables: a device failure shows as NaN in obs,
  * and kpm_sync_status (with any context of the device) reports and clears the
  * fault word. */

@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
   auto grid_wait = [&]() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); };
   auto poison = [&]() {  // NaN over the tile's outputs
     grid_wait();
-    const float nan = __int_as_float(0x7fc00000);
+    const float nan = __int_as_float(-1);  // all bits set: NaN as FP32 and, two of them, as FP64
     const float4 nan4 = make_float4(nan, nan, nan, nan);
     for (int t = threadIdx.x; t < nrow * 2 * w * NV; t += blockDim.x) {
       const int r = t / (2 * w * NV), k = t - r * (2 * w * NV);

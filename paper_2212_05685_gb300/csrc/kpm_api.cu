@@ -636,7 +636,7 @@ int kpm_destroy(kpm_ctx* ctx) {
   return KPM_OK;
 }
 
-// KPM_ETIMEDOUT / KPM_ECUDA for a fault recorded by the FP32 recursion, else
+// KPM_ETIMEDOUT / KPM_ECUDA for a fault recorded by the march kernel, else
 // 0; a recorded fault is cleared once the device is idle (the launches that
 // saw it have written NaN by then)
 static int device_fault_status(kpm_ctx* ctx) {
@@ -648,9 +648,9 @@ static int device_fault_status(kpm_ctx* ctx) {
   if ((e = clear_step_fault()) != cudaSuccess) return cuda_fail(ctx, e, "clearing the device fault word");
   if (f & 1u)
     return fail(ctx, KPM_ETIMEDOUT,
-                "a bounded wait of the FP32 recursion expired: the outputs of that launch, and of every FP32 "
+                "a bounded wait of the recursion expired: the outputs of that launch, and of every TMA-staged "
                 "recursion launch after it until this report, are NaN");
-  return fail(ctx, KPM_ECUDA, "shared memory of the FP32 recursion was not aligned for TMA: outputs are NaN");
+  return fail(ctx, KPM_ECUDA, "shared memory of the recursion was not aligned for TMA: outputs are NaN");
 }
 
 int kpm_sync_status(kpm_ctx* ctx, void* stream) {
