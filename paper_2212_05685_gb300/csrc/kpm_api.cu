@@ -1603,7 +1603,8 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
       q.residual = h[4];
       q.density_error = h[5];
       q.iterations = it + 1;
-      if (!(q.residual == q.residual) || !(q.omega == q.omega) || q.residual > 1e300) {
+      // (the word is cleared as it is read: asked once, for the first such cell)
+      if (status == KPM_OK && (!(q.residual == q.residual) || !(q.omega == q.omega) || q.residual > 1e300)) {
         status = device_fault_status(ctx);
         if (status == KPM_OK) status = fail(ctx, KPM_ENONFINITE, "non-finite order parameters in a batched cell");
       }

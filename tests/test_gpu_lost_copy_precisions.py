@@ -21,7 +21,7 @@ import torch
 from paper_2212_05685_gb300 import build, inputs, kpm
 build.build()
 ctx = kpm.kpm_create(0)
-nx, ny, M, prec = 24, 14, 512, {prec}
+nx, ny, M, prec, cells = 24, 14, 512, {prec}, {cells}
 N = nx * ny
 model = kpm.make_model(nx, ny)
 phi = torch.empty(4 * N, dtype=torch.float64, device="cuda")
@@ -43,8 +43,9 @@ def iterate():
     mu = torch.zeros(1, dtype=torch.float64, device="cuda")
     return kpm.rmft_iterate(ctx, model, opts, ro, phi, seed.clone(), mu, 1, check=False)[0]
 def batched():  # 672 Nambu rows: FP32 cells of this size run the march kernel
-    mu = torch.zeros(1, dtype=torch.float64, device="cuda")
-    return kpm.rmft_iterate_batched(ctx, [model], opts, [ro], [phi], [seed.clone()], mu, 1, check=False)[0]
+    mu = torch.zeros(cells, dtype=torch.float64, device="cuda")
+    return kpm.rmft_iterate_batched(ctx, [model] * cells, opts, [ro] * cells, [phi] * cells,
+                                    [seed.clone() for _ in range(cells)], mu, 1, check=False)[0]
 st, ref = observables()
 assert st == kpm.KPM_OK and bool(torch.isfinite(ref).all())
 kpm.kpm_inject_lost_copy(ctx, 1, 0.05)
@@ -54,7 +55,7 @@ assert bool(torch.isnan(bad[:2 * N]).all()), "densities that are not NaN"
 kpm.kpm_inject_lost_copy(ctx, 1, 0.05)
 st = iterate()
 assert st == kpm.KPM_ETIMEDOUT, ("iterate", st)
-if prec != kpm.KPM_DF64:
+if cells:  # (double-float: refused by the batched call)
     kpm.kpm_inject_lost_copy(ctx, 1, 0.05)
     st = batched()
     assert st == kpm.KPM_ETIMEDOUT, ("batched", st)
@@ -66,12 +67,14 @@ print("lost-copy path ok")
 """
 
 
-@pytest.mark.parametrize("prec", [0, 1, 2], ids=["fp64", "fp32", "df64"])
-def test_lost_copy_reads_as_nan(prec):
+# the cells after a faulted one are NaN too: the batch reports the fault, not theirs
+@pytest.mark.parametrize("prec,cells", [(0, 1), (0, 3), (1, 1), (1, 3), (2, 0)],
+                         ids=["fp64", "fp64-3-cells", "fp32", "fp32-3-cells", "df64"])
+def test_lost_copy_reads_as_nan(prec, cells):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    res = subprocess.run([sys.executable, "-c", _CHILD.format(root=root, prec=prec)], capture_output=True, text=True,
-                         timeout=300)
+    res = subprocess.run([sys.executable, "-c", _CHILD.format(root=root, prec=prec, cells=cells)], capture_output=True,
+                         text=True, timeout=300)
     assert res.returncode == 0, res.stdout + res.stderr
     assert "lost-copy path ok" in res.stdout
