@@ -27,8 +27,7 @@ struct kpm_ctx {
 
   // scratch (owned)
   void* slab[4] = {nullptr, nullptr, nullptr, nullptr};  // two, or four for several steps per launch
-  int slab_n = 0;
-  size_t slab_bytes = 0;
+  size_t slab_bytes[4] = {0, 0, 0, 0};
   double2* xi = nullptr;  // probing phases conj(xi_J) of the current pass
   size_t xi_bytes = 0;
   // LDOS: diagonal-moment record, coefficient matrix, weights, frequencies, cuBLAS handle
@@ -201,25 +200,49 @@ void drop_batch_graph(kpm_ctx* ctx) {
   ctx->bkey.clear();
 }
 
-// at least `n` recursion slabs of `bytes` (the first two serve every pass)
-int ensure_slabs(kpm_ctx* ctx, size_t bytes, int n) {
-  if (ctx->slab_bytes >= bytes && ctx->slab_n >= n) return KPM_OK;
-  drop_graph(ctx);
-  for (int k = 0; k < 4; ++k) {
-    if (ctx->slab[k]) cudaFree(ctx->slab[k]);
+// free slabs [n, 4); true if there were any
+bool release_slabs(kpm_ctx* ctx, int n) {
+  bool any = false;
+  for (int k = n; k < 4; ++k) {
+    if (!ctx->slab[k]) continue;
+    if (!any) drop_graph(ctx);
+    any = true;
+    cudaFree(ctx->slab[k]);
     ctx->slab[k] = nullptr;
+    ctx->slab_bytes[k] = 0;
   }
-  ctx->slab_bytes = 0;
-  ctx->slab_n = 0;
-  for (int k = 0; k < n; ++k) {
-    if (cudaMalloc(&ctx->slab[k], bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(ctx, KPM_ENOMEM, "cudaMalloc of the recursion slabs failed");
+  return any;
+}
+
+// `n` recursion slabs of at least `bytes` (the first two serve every pass).  Slabs only
+// grow, each by itself, and those beyond n stay, so that passes of different
+// precision and steps per launch in turn neither free nor allocate, nor lose the
+// iteration graph, as long as the budget holds what they need together.
+int ensure_slabs(kpm_ctx* ctx, size_t bytes, int n) {
+  bool grow = false;
+  uint64_t held = 0;
+  for (int k = 0; k < 4; ++k) {
+    grow = grow || (k < n && ctx->slab_bytes[k] < bytes);
+    held += k < n ? std::max(ctx->slab_bytes[k], bytes) : ctx->slab_bytes[k];
+  }
+  if (!grow) return KPM_OK;
+  if (held > ctx->budget) release_slabs(ctx, 0);
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    bool ok = true;
+    for (int k = 0; k < n && ok; ++k) {
+      if (ctx->slab_bytes[k] >= bytes) continue;
+      drop_graph(ctx);
+      if (ctx->slab[k]) cudaFree(ctx->slab[k]);
+      ctx->slab_bytes[k] = 0;
+      ok = cudaMalloc(&ctx->slab[k], bytes) == cudaSuccess;
+      if (ok) ctx->slab_bytes[k] = bytes;
+      else ctx->slab[k] = nullptr;
     }
+    if (ok) return KPM_OK;
+    cudaGetLastError();
+    release_slabs(ctx, 0);  // the device may hold what is needed now, if not what is kept
   }
-  ctx->slab_bytes = bytes;
-  ctx->slab_n = n;
-  return KPM_OK;
+  return fail(ctx, KPM_ENOMEM, "cudaMalloc of the recursion slabs failed");
 }
 
 int ensure_site_scratch(kpm_ctx* ctx, int N) {
