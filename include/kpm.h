@@ -118,7 +118,8 @@ typedef struct {
  * launch than by default, where the lattice allows it (default: one step per
  * launch while the slabs stay in L2 or the budget holds no four slabs, else
  * two; every choice gives the same bits; kpm_autotune picks the faster).
- * Launches of several steps need four slabs instead of two. */
+ * Launches of several steps need four slabs instead of two; where the device has no
+ * memory for four, a pass takes one step per launch on two. */
 #define KPM_FLAG_DOUBLE_STEP 1
 /* kpm_opts.flags: particle-hole half pass.  Only the N unit columns (j, up)
  * are propagated; the spin-down observables and the other half of the grand

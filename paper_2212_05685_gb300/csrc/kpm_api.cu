@@ -28,6 +28,7 @@ struct kpm_ctx {
   // scratch (owned)
   void* slab[4] = {nullptr, nullptr, nullptr, nullptr};  // two, or four for several steps per launch
   size_t slab_bytes[4] = {0, 0, 0, 0};
+  bool oom = false;  // the last KPM_ENOMEM was for want of device memory
   double2* xi = nullptr;  // probing phases conj(xi_J) of the current pass
   size_t xi_bytes = 0;
   // LDOS: diagonal-moment record, coefficient matrix, weights, frequencies, cuBLAS handle
@@ -180,6 +181,7 @@ int ensure(kpm_ctx* ctx, T** p, size_t* have, size_t need_bytes) {
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
+    ctx->oom = e == cudaErrorMemoryAllocation;
     return fail(ctx, KPM_ENOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
   }
   *have = need_bytes;
@@ -228,19 +230,40 @@ int ensure_slabs(kpm_ctx* ctx, size_t bytes, int n) {
   if (!grow) return KPM_OK;
   if (held > ctx->budget) release_slabs(ctx, 0);
   for (int attempt = 0; attempt < 2; ++attempt) {
-    bool ok = true;
-    for (int k = 0; k < n && ok; ++k) {
+    cudaError_t e = cudaSuccess;
+    bool fresh[4] = {false, false, false, false};
+    for (int k = 0; k < n && e == cudaSuccess; ++k) {
       if (ctx->slab_bytes[k] >= bytes) continue;
-      drop_graph(ctx);
-      if (ctx->slab[k]) cudaFree(ctx->slab[k]);
-      ctx->slab_bytes[k] = 0;
-      ok = cudaMalloc(&ctx->slab[k], bytes) == cudaSuccess;
-      if (ok) ctx->slab_bytes[k] = bytes;
-      else ctx->slab[k] = nullptr;
+      if (ctx->slab[k]) {
+        drop_graph(ctx);
+        cudaFree(ctx->slab[k]);
+        ctx->slab_bytes[k] = 0;
+      }
+      if ((e = cudaMalloc(&ctx->slab[k], bytes)) != cudaSuccess) {
+        ctx->slab[k] = nullptr;
+        break;
+      }
+      ctx->slab_bytes[k] = bytes;
+      fresh[k] = true;
     }
-    if (ok) return KPM_OK;
+    if (e == cudaSuccess) {
+      drop_graph(ctx);
+      return KPM_OK;
+    }
     cudaGetLastError();
-    release_slabs(ctx, 0);  // the device may hold what is needed now, if not what is kept
+    ctx->oom = e == cudaErrorMemoryAllocation;
+    // what was held stays, unless the pass could do with less of it: then once more
+    bool excess = false;
+    for (int k = 0; k < 4; ++k) {
+      if (fresh[k]) {
+        cudaFree(ctx->slab[k]);
+        ctx->slab[k] = nullptr;
+        ctx->slab_bytes[k] = 0;
+      }
+      excess = excess || ctx->slab_bytes[k] > (k < n ? bytes : 0);
+    }
+    if (!excess || !ctx->oom) break;
+    release_slabs(ctx, 0);
   }
   return fail(ctx, KPM_ENOMEM, "cudaMalloc of the recursion slabs failed");
 }
@@ -281,8 +304,9 @@ int64_t balanced_width(int64_t D, int64_t width) {
   return (D + n - 1) / n;
 }
 
-// single: FP32 unit vectors one step per launch (a caller that needs every vector)
-int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp, bool single = false) {
+// single: FP32 unit vectors one step per launch (a caller that needs every vector);
+// slabs: two hold the plan to one step per launch, four leave it the choice
+int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp, bool single = false, int slabs = 4) {
   if (!o) return fail(ctx, KPM_EINVAL, "opts is null");
   if (o->M < 1) return fail(ctx, KPM_EINVAL, "M must be >= 1");
   if (o->precision != KPM_FP32 && o->precision != KPM_FP64 && o->precision != KPM_DF64)
@@ -312,7 +336,8 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
       return fail(ctx, KPM_EINVAL, "KPM_FLAG_PH_HALF and a site range do not combine");
   }
   const bool march = o->precision == KPM_FP32 || pp_ == 0;  // (FP64 and double-float probing: the one-step kernels)
-  const bool deeper = o->precision == KPM_FP32 && pp_ == 0 && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
+  const bool deeper =
+      o->precision == KPM_FP32 && pp_ == 0 && slabs >= 4 && (o->flags & KPM_FLAG_DOUBLE_STEP) && o->M > 2;
   const int js = (o->flags & KPM_FLAG_PH_HALF) ? 1 : 0;
   // start vectors of the pass: unit columns (those of the site range), or R = 2 p^2 probing vectors
   pp->c0 = pp->ranged ? 2 * (int64_t)pp->sb : 0;
@@ -320,14 +345,14 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
   const int64_t ncols = pp->c1 - pp->c0;
   // slab width: as asked, else as many columns as fit the budget; several steps per
   // launch need four slabs, a default that does not fit them takes one step
-  auto width_of = [&](int slabs) {
+  auto width_of = [&](int n) {
     if (o->block_width > 0) return std::min<int64_t>(o->block_width, ncols);
-    const int64_t fit = (int64_t)(ctx->budget / ((uint64_t)slabs * (uint64_t)D * pp->elem));
+    const int64_t fit = (int64_t)(ctx->budget / ((uint64_t)n * (uint64_t)D * pp->elem));
     return balanced_width(ncols, std::min<int64_t>(ncols, std::max<int64_t>(fit, 1)));
   };
   int64_t width = width_of(2);
   int steps = march ? (single || pp_ > 0 || o->precision != KPM_FP32 ? 1 : march_steps(m->nx, m->ny, width)) : 0;
-  if (steps > 1 && (o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
+  if (steps > 1 && (slabs < 4 || o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
   if (deeper) ++steps;
   if (steps > 1) width = width_of(4);
   pp->cheb = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows, steps,
@@ -383,6 +408,25 @@ int ensure_pass_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, con
   cudaError_t e = cheb_prepare(pp.cheb, o->precision);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cheb_prepare");
   return KPM_OK;
+}
+
+// plan of a pass and its scratch, with what else the caller holds during it (`extra`:
+// a status, for the plan in *pp).  Where the device does not hold four slabs, or two
+// beside slabs kept from other passes, those beyond two go and the pass takes one step per launch.
+template <typename Extra>
+int plan_with_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp, bool single, Extra extra) {
+  for (int slabs = 4;; slabs = 2) {
+    int r = plan_pass(ctx, m, o, pp, single, slabs);
+    if (r) return r;
+    ctx->oom = false;
+    r = ensure_pass_scratch(ctx, m, o, *pp);
+    if (!r) r = extra();
+    if (r != KPM_ENOMEM || !ctx->oom || slabs == 2) return r;
+    if (!release_slabs(ctx, 2) && pp->cheb.mk.ns <= 1) return r;
+  }
+}
+int plan_with_scratch(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp, bool single = false) {
+  return plan_with_scratch(ctx, m, o, pp, single, [] { return (int)KPM_OK; });
 }
 
 // V_1 .. V_{M-1} of a unit-vector slab by single steps of the march kernel, from V_0 in
@@ -767,22 +811,27 @@ int kpm_observables(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, 
     return r;
   if (omega && (r = check_dev(ctx, omega, "omega"))) return r;
   DeviceGuard g(ctx->device);
+  if (!opts) return fail(ctx, KPM_EINVAL, "opts is null");
+  const int N = model->nx * model->ny;
+  const bool keep = (opts->flags & KPM_FLAG_KEEP_TAIL) && opts->M >= 2;
+  const bool tail_ok = opts->precision != KPM_DF64 && !opts->probe_p && !(opts->flags & KPM_FLAG_PH_HALF);
   PassPlan pp;
-  if ((r = plan_pass(ctx, model, opts, &pp))) return r;
-  if ((r = ensure_pass_scratch(ctx, model, opts, pp))) return r;
+  r = plan_with_scratch(ctx, model, opts, &pp, false, [&] {
+    if (!keep || !tail_ok) return (int)KPM_OK;
+    ctx->tail_valid = false;
+    const size_t vec = (size_t)pp.cheb.D * pp.cheb.ldv * pp.elem;
+    const int64_t nslab = (pp.c1 - pp.c0 + pp.width - 1) / pp.width;
+    const int e = ensure(ctx, &ctx->tail, &ctx->tail_bytes, 2 * (size_t)nslab * vec);
+    return e ? e : ensure(ctx, &ctx->tail_in, &ctx->tail_in_bytes, (26 * (size_t)N + 2) * sizeof(double));
+  });
+  if (r) return r;
   if (opts->flags & KPM_FLAG_PH_HALF) {
     if ((r = check_ph_sector(ctx, model, fields, ab, (cudaStream_t)stream))) return r;
   }
   void* tail = nullptr;
   ctx->tail_valid = false;
-  if ((opts->flags & KPM_FLAG_KEEP_TAIL) && opts->M >= 2) {
-    if (opts->precision == KPM_DF64 || opts->probe_p || (opts->flags & KPM_FLAG_PH_HALF))
-      return fail(ctx, KPM_EINVAL, "KPM_FLAG_KEEP_TAIL: FP32 or FP64 unit-vector passes only");
-    const int N = model->nx * model->ny;
-    const size_t vec = (size_t)pp.cheb.D * pp.cheb.ldv * pp.elem;
-    const int64_t nslab = (pp.c1 - pp.c0 + pp.width - 1) / pp.width;
-    if ((r = ensure(ctx, &ctx->tail, &ctx->tail_bytes, 2 * (size_t)nslab * vec))) return r;
-    if ((r = ensure(ctx, &ctx->tail_in, &ctx->tail_in_bytes, (26 * (size_t)N + 2) * sizeof(double)))) return r;
+  if (keep) {
+    if (!tail_ok) return fail(ctx, KPM_EINVAL, "KPM_FLAG_KEEP_TAIL: FP32 or FP64 unit-vector passes only");
     cudaStream_t s = (cudaStream_t)stream;
     KPM_CU(cudaMemcpyAsync(ctx->tail_in, fields, 26 * (size_t)N * sizeof(double), cudaMemcpyDeviceToDevice, s));
     KPM_CU(cudaMemcpyAsync(ctx->tail_in + 26 * (size_t)N, ab, 2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -870,7 +919,7 @@ int rmft_iterate(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
   if ((r = plan_pass(ctx, model, opts, &pp))) return r;
   if (pp.ranged) return fail(ctx, KPM_EINVAL, "rmft_iterate needs the whole lattice (site range 0, 0)");
   if ((r = ensure_site_scratch(ctx, N))) return r;
-  if ((r = ensure_pass_scratch(ctx, model, opts, pp))) return r;
+  if ((r = plan_with_scratch(ctx, model, opts, &pp))) return r;
   if ((r = ensure_misc(ctx))) return r;
   AndersonState an;
   if (ropts->anderson > 0) {
@@ -1058,22 +1107,25 @@ int kpm_backward(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
     o.block_width = (int)balanced_width(ncol, std::max<int64_t>(1, std::min<int64_t>(ncol, fit)));
   }
   PassPlan pp;
-  if ((r = plan_pass(ctx, model, &o, &pp, true))) return r;
-  if ((r = ensure_pass_scratch(ctx, model, &o, pp))) return r;
   const ChebPlan& p = pp.cheb;
-  const size_t vbytes = (size_t)D * p.ldv * elem;
+  size_t vbytes = 0, gbytes = 0;
+  int groups = 0;
+  r = plan_with_scratch(ctx, model, &o, &pp, true, [&] {
+    vbytes = (size_t)D * p.ldv * elem;
+    groups = grad_groups(p, o.precision);
+    gbytes = (size_t)D * 13 * sizeof(double2);  // G, then the column sets' partial sums
+    int e = ensure(ctx, &ctx->bwd, &ctx->bwd_bytes, vbytes * (size_t)nvec);
+    if (!e) e = ensure(ctx, &ctx->Gacc, &ctx->Gacc_bytes, gbytes * (size_t)(groups + 1));
+    return e ? e : ensure(ctx, &ctx->wseed, &ctx->wseed_bytes, (size_t)D * kSlots * sizeof(double2));
+  });
+  if (r) return r;
   if (use_tail) {
     // the tail is read slab by slab: only with the forward pass's exact slabs
     const int64_t nslab = (pp.c1 - pp.c0 + pp.width - 1) / pp.width;
     use_tail = pp.width == ctx->tail_width && pp.c0 == ctx->tail_c0 && pp.c1 == ctx->tail_c1 &&
                (size_t)(2 * nslab) * vbytes <= ctx->tail_bytes;
   }
-  if ((r = ensure(ctx, &ctx->bwd, &ctx->bwd_bytes, vbytes * (size_t)nvec))) return r;
-  const int groups = grad_groups(p, o.precision);
-  const size_t gbytes = (size_t)D * 13 * sizeof(double2);  // G, then the column sets' partial sums
-  if ((r = ensure(ctx, &ctx->Gacc, &ctx->Gacc_bytes, gbytes * (size_t)(groups + 1)))) return r;
   double2* Gpart = ctx->Gacc + (size_t)D * 13;
-  if ((r = ensure(ctx, &ctx->wseed, &ctx->wseed_bytes, (size_t)D * kSlots * sizeof(double2)))) return r;
   char* base = static_cast<char*>(ctx->bwd);
   auto ckpt = [&](int k) { return (void*)(base + vbytes * (size_t)k); };
   auto segv = [&](int j) { return (void*)(base + vbytes * (size_t)(2 * K + j)); };
@@ -1225,13 +1277,13 @@ int kpm_ldos(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, const d
   kpm_opts o = *opts;
   o.flags &= ~KPM_FLAG_DOUBLE_STEP;  // one step per launch
   if ((r = ensure_site_scratch(ctx, N))) return r;
-  PassPlan pp;
-  if ((r = plan_pass(ctx, model, &o, &pp))) return r;
-  if ((r = ensure_pass_scratch(ctx, model, &o, pp))) return r;
   // scratch: record M x D, coefficients 2 x n_omega x M, weights 2N, frequencies n_omega
   const size_t rec_n = (size_t)M * D, c_n = 2 * (size_t)n_omega * M;
   const size_t need = (rec_n + c_n + 2 * (size_t)N + (size_t)n_omega) * sizeof(double);
-  if ((r = ensure(ctx, &ctx->ldos_buf, &ctx->ldos_buf_bytes, need))) return r;
+  PassPlan pp;
+  if ((r = plan_with_scratch(ctx, model, &o, &pp, false,
+                             [&] { return ensure(ctx, &ctx->ldos_buf, &ctx->ldos_buf_bytes, need); })))
+    return r;
   double* rec = ctx->ldos_buf;
   double* C = rec + rec_n;
   double* wgt = C + c_n;
@@ -1331,8 +1383,11 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
     for (size_t k = 0; k < members.size(); ++k)
       if (!persist[k]) march_slab = std::max(march_slab, (size_t)plans[k].D * plans[k].ldv * elem);
     r = KPM_OK;
-    for (int k = 0; k < 2 && r == KPM_OK && march_slab > 0; ++k)
+    for (int k = 0; k < 2 && r == KPM_OK && march_slab > 0; ++k) {
       r = ensure(ctx, &ctx->bslab[k], &ctx->bslab_bytes[k], march_slab);
+      if (r == KPM_ENOMEM && ctx->oom && release_slabs(ctx, 2))
+        r = ensure(ctx, &ctx->bslab[k], &ctx->bslab_bytes[k], march_slab);
+    }
     if (r == KPM_OK) break;
     if (!small) return r;
   }
@@ -1725,8 +1780,8 @@ int kpm_autotune(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
       for (int bk = 0; bk < nband && !r; ++bk) {
         o.band_rows = bands[bk];
         o.M = Mt2;
-        if (bk && plan_pass(ctx, model, &o, &pp) != KPM_OK) continue;
-        if ((r = ensure_pass_scratch(ctx, model, &o, pp))) break;
+        if ((r = plan_with_scratch(ctx, model, &o, &pp))) break;
+        if (mode && !pp.deeper) continue;  // the device does not hold its slabs
         // one warm-up pass, then one timed pass at each trial order
         if ((r = enqueue_pass(ctx, model, &o, pp, fields, ab, ctx->obs, nullptr, s))) break;
         float ms[2] = {0.f, 0.f};

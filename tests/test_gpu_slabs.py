@@ -81,3 +81,50 @@ def test_kept_slabs_stay_within_the_budget(kpm):
             assert all(np.array_equal(a, b) for a, b in zip(got, first))
     finally:
         kpm.kpm_destroy(ctx)
+
+
+def _room(nbytes):
+    free, _ = torch.cuda.mem_get_info()
+    if free < nbytes:
+        pytest.skip("needs a device with that much free memory")
+
+
+def test_two_slabs_where_four_do_not_fit_the_device(kpm):
+    """220x220 under a budget above the device's memory: four slabs of 75 GB do not fit it,
+    two do.  The pass runs one step per launch on two, with the bits of narrow slabs, and so does
+    the next one."""
+    torch.cuda.empty_cache()
+    _room(200 << 30)
+    ctx = kpm.kpm_create(0)
+    try:
+        cell = _cell(kpm, ctx, 220, 220)
+        ref = _pass(kpm, ctx, cell, 3, kpm.KPM_FP32, block_width=4096)
+        kpm.kpm_set_scratch_budget(ctx, 400 << 30)
+        for flags in (0, kpm.KPM_FLAG_DOUBLE_STEP, 0):
+            assert np.array_equal(_pass(kpm, ctx, cell, 3, kpm.KPM_FP32, flags=flags), ref)
+            assert torch.cuda.mem_get_info()[0] > 100 << 30  # two slabs of 75 GB of 284
+    finally:
+        kpm.kpm_destroy(ctx)
+
+
+def test_backward_after_a_pass_on_four_slabs(kpm):
+    """220x196: the forward pass's four slabs of 60 GB fit the device, the backward pass's two
+    vectors beside them do not; it runs on two of the slabs."""
+    torch.cuda.empty_cache()
+    _room(255 << 30)
+    ctx = kpm.kpm_create(0)
+    try:
+        cell = model, fields, ab = _cell(kpm, ctx, 220, 196)
+        go = torch.ones_like(fields)
+        opts = kpm.make_opts(3, kpm.KPM_FP32)
+        want, got = torch.empty_like(fields), torch.empty_like(fields)
+        narrow = kpm.make_opts(3, kpm.KPM_FP32, block_width=8192)
+        kpm.kpm_backward(ctx, model, narrow, fields, ab, go, 0.0, want, ckpt_every=kpm.KPM_REGENERATE)
+        kpm.kpm_set_scratch_budget(ctx, 400 << 30)
+        _pass(kpm, ctx, cell, 3, kpm.KPM_FP32)
+        kpm.kpm_backward(ctx, model, opts, fields, ab, go, 0.0, got, ckpt_every=kpm.KPM_REGENERATE)
+        assert kpm.kpm_sync_status(ctx) == kpm.KPM_OK
+        # the sums over the columns are split at other places: FP32 rounding of their products
+        assert float((got - want).abs().max()) < 1e-5 * float(want.abs().max())
+    finally:
+        kpm.kpm_destroy(ctx)
