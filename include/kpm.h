@@ -116,8 +116,9 @@ typedef struct {
 
 /* kpm_opts.flags: run the FP32 recursion on unit vectors one step more per
  * launch than by default, where the lattice allows it (default: one step per
- * launch while the slabs stay in L2 or the budget holds no four slabs, else
- * two; every choice gives the same bits; kpm_autotune picks the faster).
+ * launch while the slabs stay in L2, else two where they pay at the width of which
+ * the budget holds four slabs; every choice gives the same bits; kpm_autotune picks the
+ * faster).
  * Launches of several steps need four slabs instead of two; where the device has no
  * memory for four, a pass takes one step per launch on two. */
 #define KPM_FLAG_DOUBLE_STEP 1

@@ -343,16 +343,23 @@ int plan_pass(kpm_ctx* ctx, const kpm_model* m, const kpm_opts* o, PassPlan* pp,
   pp->c0 = pp->ranged ? 2 * (int64_t)pp->sb : 0;
   pp->c1 = pp->ranged ? 2 * (int64_t)pp->se : (pp_ > 0 ? std::min<int64_t>(D, 2 * (int64_t)pp_ * pp_) : (D >> js));
   const int64_t ncols = pp->c1 - pp->c0;
-  // slab width: as asked, else as many columns as fit the budget; several steps per
-  // launch need four slabs, a default that does not fit them takes one step
+  // slab width: as asked, else as many columns as fit the budget
   auto width_of = [&](int n) {
     if (o->block_width > 0) return std::min<int64_t>(o->block_width, ncols);
     const int64_t fit = (int64_t)(ctx->budget / ((uint64_t)n * (uint64_t)D * pp->elem));
     return balanced_width(ncols, std::min<int64_t>(ncols, std::max<int64_t>(fit, 1)));
   };
   int64_t width = width_of(2);
-  int steps = march ? (single || pp_ > 0 || o->precision != KPM_FP32 ? 1 : march_steps(m->nx, m->ny, width)) : 0;
-  if (steps > 1 && (slabs < 4 || o->M < 3 || 4 * (uint64_t)D * width_of(4) * pp->elem > ctx->budget)) steps = 1;
+  int steps = march ? 1 : 0;
+  if (o->precision == KPM_FP32 && pp_ == 0 && !single && slabs >= 4 && o->M >= 3 &&
+      march_steps(m->nx, m->ny, width) > 1) {
+    // Two steps per launch take four slabs, which narrows the default width where the budget
+    // does not hold four of this one: only if they pay at the width that will run, and
+    // if the budget holds four of a width that was asked for.  50x34 under 200 MB, M = 256: two steps
+    // on four slabs of 1700 columns, two of which stay in L2, 13.9 ms; one step on two of 3400 11.3.
+    const int64_t w4 = width_of(4);
+    if (4 * (uint64_t)D * w4 * pp->elem <= ctx->budget && (w4 == width || march_steps(m->nx, m->ny, w4) > 1)) steps = 2;
+  }
   if (deeper) ++steps;
   if (steps > 1) width = width_of(4);
   pp->cheb = plan_cheb(m->nx, m->ny, width, o->precision, o->cols_per_block, o->band_rows, steps,
