@@ -1405,9 +1405,11 @@ int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
   return band_rows_candidates(ny, ldv / march_cols(p.el) * p.ntile, out, maxn, per_sm * kSMs, start);
 }
 
-// Geometry of a march launch: the whole lattice row per CTA where its threads
-// fit, else the fewest equal tiles; then the deepest rings that fit shared
+// Geometry of a march launch: the whole lattice row per CTA where its threads and rings
+// fit, else the fewest equal tiles that do; the deepest rings that fit shared
 // memory (several steps: eight rows each), and the band height of the wave model.
+// (Two steps in tiles of 26 sites do not fit: 104x104 in five tiles of 21, M = 65, 96.6 ms, one
+// step 113.2; 180x60 in eight of 23, M = 33, 53.0 and 56.3.)
 MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows, int el = kElF32) {
   MarchPlan p;
   p.el = el;
@@ -1417,42 +1419,41 @@ MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows, int el 
     for (int s = 0; s < ns; ++s) n += ((full ? nx : tx + 2 * (ns - 1 - s)) * nv + 31) / 32;
     return n;
   };
-  if (warps(nx, true) * 32 <= kMarchThreads) {
+  // A set of rows is issued once the last stage has finished the row `lag` before it;
+  // single step: row i + 2 of V_m then takes the place of one that the stage and the
+  // sums have done with in a ring of lag + 2 rows
+  // (a row of double-float or FP64 takes as long as its copy: four are enough)
+  auto fits = [&](int tx, bool full) {
+    p.warps = warps(tx, full);
+    if (p.warps * 32 > kMarchThreads) return false;
+    p.wrow = full ? nx : tx + 2 * ns;
+    p.crowb = (p.wrow * march_entry_bytes(el) + 127) / 128 * 128;
+    for (int lag = el == kElF32 ? 8 : 4; lag >= (ns == 1 ? 2 : 8); --lag) {
+      p.lag = lag;
+      p.rv = ns == 1 ? lag + 2 : kMarchRows;
+      p.rp = p.rc = ns == 1 ? lag : kMarchRows;
+      p.rs = kMarchRows;
+      p.smem = 32 * (size_t)nv * p.wrow * (p.rv + p.rp + (ns - 1) * p.rs) + (size_t)p.crowb * p.rc +
+               8 * (size_t)kMarchBars * (1 + ns) + 16;
+      if (p.smem <= kSmemLimit) return true;
+    }
+    return false;
+  };
+  if (fits(nx, true)) {
     p.full = 1;
     p.ntile = 1;
     p.tx = nx;
   } else {
-    for (int nt = 2; nt <= nx; ++nt) {
+    for (int nt = 2; nt <= nx && p.ntile == 0; ++nt) {
       const int tx = (nx + nt - 1) / nt;
       const int last = nx - (nt - 1) * tx;
-      if (warps(tx, false) * 32 <= kMarchThreads && last >= ns && tx >= ns) {
-        p.ntile = nt;
-        p.tx = tx;
-        break;
-      }
+      if (last < ns || tx < ns || !fits(tx, false)) continue;
+      p.ntile = nt;
+      p.tx = tx;
     }
     if (p.ntile == 0) return p;
   }
-  p.warps = warps(p.tx, p.full);
-  p.wrow = p.full ? nx : p.tx + 2 * ns;
-  p.crowb = (p.wrow * march_entry_bytes(el) + 127) / 128 * 128;
-  // a set of rows is issued once the last stage has finished the row `lag` before it;
-  // single step: row i + 2 of V_m then takes the place of one that the stage and the
-  // sums have done with in a ring of lag + 2 rows
-  // (a row of double-float or FP64 takes as long as its copy: four are enough)
-  for (int lag = el == kElF32 ? 8 : 4; lag >= (ns == 1 ? 2 : 8); --lag) {
-    p.lag = lag;
-    p.rv = ns == 1 ? lag + 2 : kMarchRows;
-    p.rp = p.rc = ns == 1 ? lag : kMarchRows;
-    p.rs = kMarchRows;
-    p.smem = 32 * (size_t)nv * p.wrow * (p.rv + p.rp + (ns - 1) * p.rs) + (size_t)p.crowb * p.rc +
-             8 * (size_t)kMarchBars * (1 + ns) + 16;
-    if (p.smem <= kSmemLimit) {
-      p.ns = ns;
-      break;
-    }
-  }
-  if (p.ns == 0) return p;
+  p.ns = ns;
   int best = ny;
   march_bands(p, ny, ldv, &best, 1);
   p.ylen = band_rows > 0 ? std::min(band_rows, ny) : best;
