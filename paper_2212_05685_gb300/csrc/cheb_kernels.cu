@@ -1394,14 +1394,16 @@ cudaError_t march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, con
 
 namespace {
 // band heights of a march launch: as many CTAs per SM as registers and shared memory
-// take; a CTA's start (barriers, first copies) costs about five rows (one of double-float
-// or FP64), and a launch of several steps computes two more rows for every step but the last
+// take; a CTA's start (barriers, first copies) costs about five rows (one of double-float;
+// 0.3 of FP64, whose rows are bound by the FP64 pipe: passes of M = 65 with 1.0 and 0.3, ms:
+// 40x11 5.71 and 4.97, 45x10 6.21 and 5.43, 30x21 11.71 and 10.61, 104x7 14.33 and 13.27),
+// and a launch of several steps computes two more rows for every step but the last
 int march_per_sm(const MarchPlan& p) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(16 / p.warps, (int64_t)(228 * 1024) / (int64_t)(p.smem + 1024)));
 }
 int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
   const int per_sm = march_per_sm(p);
-  const double start = p.el == kElF32 ? 5.0 + 2.0 * (p.ns - 1) : 1.0;
+  const double start = p.el == kElF32 ? 5.0 + 2.0 * (p.ns - 1) : p.el == kElDF ? 1.0 : 0.3;
   return band_rows_candidates(ny, ldv / march_cols(p.el) * p.ntile, out, maxn, per_sm * kSMs, start);
 }
 
