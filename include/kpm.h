@@ -314,7 +314,8 @@ int kpm_autotune(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, con
 
 /* Batched self-consistency (cells of uneven size, doping and field): up to
  * n_iter iterations of rmft_iterate's loop for ncell independent cells,
- * replayed as CUDA graphs.  FP32: cells of up to 640 Nambu rows run the persistent
+ * replayed as CUDA graphs.  FP32: cells of up to 640 Nambu rows (704 or 720 of some
+ * shapes) run the persistent
  * recursion: one launch per iteration for all of them, in which a cluster of 8
  * CTAs holds a 16-column chunk of one cell on chip for all M moments (work
  * items longest first); larger cells run one after the other on the march

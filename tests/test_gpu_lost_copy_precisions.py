@@ -21,7 +21,7 @@ import torch
 from paper_2212_05685_gb300 import build, inputs, kpm
 build.build()
 ctx = kpm.kpm_create(0)
-nx, ny, M, prec, cells = 24, 14, 512, {prec}, {cells}
+nx, ny, M, prec, cells = 32, 16, 512, {prec}, {cells}
 N = nx * ny
 model = kpm.make_model(nx, ny)
 phi = torch.empty(4 * N, dtype=torch.float64, device="cuda")
@@ -42,7 +42,7 @@ def observables():
 def iterate():
     mu = torch.zeros(1, dtype=torch.float64, device="cuda")
     return kpm.rmft_iterate(ctx, model, opts, ro, phi, seed.clone(), mu, 1, check=False)[0]
-def batched():  # 672 Nambu rows: FP32 cells of this size run the march kernel
+def batched():  # 1024 Nambu rows: FP32 cells of this size run the march kernel
     mu = torch.zeros(cells, dtype=torch.float64, device="cuda")
     return kpm.rmft_iterate_batched(ctx, [model] * cells, opts, [ro] * cells, [phi] * cells,
                                     [seed.clone() for _ in range(cells)], mu, 1, check=False)[0]
