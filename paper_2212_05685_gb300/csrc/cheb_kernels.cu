@@ -591,29 +591,25 @@ __device__ __forceinline__ void stencil_2site(const float4* wm, const float4* w0
 }
 
 // moment sums acc[J][s] += a V[K_s(J), J] for the columns of the chunk whose
-// own site lies in lattice row y; wm, w0, wp hold rows y-1, y, y+1
+// own site lies in lattice row y; wm, w0, wp hold rows y-1, y, y+1 (unit vectors of a full
+// pass: FP32 probing and half passes run the march kernel)
 template <int CB>
 __device__ __forceinline__ void moment_sums(const float4* wm, const float4* w0, const float4* wp, int nx, int y,
-                                            int64_t D, const ColMap& cmap, int64_t cb0, int m, double cm, double co,
+                                            int64_t D, int64_t s0, int m, double cm, double co,
                                             double2* __restrict__ acc) {
   constexpr int NV = CB / 2;
   constexpr int RS = 2 * NV;
-  SourceRange sr;
-  const int items = source_items(cmap, nx, y, cb0, CB, sr);
-  for (int t = threadIdx.x; t < items; t += blockDim.x) {
-    int64_t J;
-    int c, s;
-    double2 wgt;
-    if (!source_item(cmap, sr, t, y, nx, D, cb0, CB, J, c, s, wgt)) continue;
-    const int64_t j = J >> 1;
+  for (int t = threadIdx.x; t < CB * kSlots; t += blockDim.x) {
+    const int c = t / kSlots, s = t - c * kSlots;
+    const int64_t J = s0 + c, j = J >> 1;
+    if (J >= D || j / nx != y) continue;
     const int beta = (int)(J & 1);
     const int xsl = wrapi((int)(j % nx) + kSlotDx[s], nx);
     const int dy = kSlotDy[s];
     const float4* w = dy < 0 ? wm : (dy > 0 ? wp : w0);
     const int al = kSlotFlip[s] ? 1 - beta : beta;
     const float2 val = pair_elem(w + xsl * RS + al * NV, c);
-    acc_add(acc + J * kSlots + s, s == kSlots - 1 ? co : cm, wgt, (double)val.x, (double)val.y);
-    if (s == 0 && cmap.rec) record_diag(cmap, D, m, J, wgt, (double)val.x, (double)val.y);
+    acc_add_unit(acc + J * kSlots + s, s == kSlots - 1 ? co : cm, (double)val.x, (double)val.y);
   }
 }
 
@@ -623,7 +619,7 @@ __device__ __forceinline__ void moment_sums(const float4* wm, const float4* w0, 
 template <int CB, int MODE>
 __device__ __forceinline__ void f32_step_body(int nx, int ny, int64_t D, int64_t ldv, int ylen,
                                               const float2* __restrict__ table, const float4* __restrict__ Vcur,
-                                              const float4* Vprev, float4* Vout, ColMap cmap,
+                                              const float4* Vprev, float4* Vout, int64_t s0,
                                               double2* __restrict__ acc,
                                               const double* __restrict__ am, const double* __restrict__ ao, int m) {
   constexpr int NV = CB / 2;   // float4 (column pairs) per Nambu row of the chunk
@@ -650,13 +646,10 @@ __device__ __forceinline__ void f32_step_body(int nx, int ny, int64_t D, int64_t
   // rows of the chunk's own sites: only there are moment sums due
   int yj_lo = ny, yj_hi = -1;
   {
-    const int64_t clo = cmap.s0 + cb0, chi = min(D >> cmap.js, cmap.s0 + cb0 + CB) - 1;
-    if (cmap.probe_p) {  // every lattice row holds sources of every colour class
-      yj_lo = 0;
-      yj_hi = ny - 1;
-    } else if (chi >= clo) {
-      yj_lo = (int)(((clo << cmap.js) >> 1) / nx);
-      yj_hi = (int)(((chi << cmap.js) >> 1) / nx);
+    const int64_t clo = s0 + cb0, chi = min(D, s0 + cb0 + CB) - 1;
+    if (chi >= clo) {
+      yj_lo = (int)((clo >> 1) / nx);
+      yj_hi = (int)((chi >> 1) / nx);
     }
   }
 
@@ -732,7 +725,7 @@ __device__ __forceinline__ void f32_step_body(int nx, int ny, int64_t D, int64_t
     }
 
     if (MODE == 1 && acc != nullptr && y >= yj_lo && y <= yj_hi)
-      moment_sums<CB>(wm - v, w0 - v, wp - v, nx, y, D, cmap, cb0, m, am[m], ao[m], acc);
+      moment_sums<CB>(wm - v, w0 - v, wp - v, nx, y, D, s0 + cb0, m, am[m], ao[m], acc);
     bm = b0;
     bc = bc + 1 == 3 ? 0 : bc + 1;
     if (MODE == 1) {
@@ -748,10 +741,10 @@ __device__ __forceinline__ void f32_step_body(int nx, int ny, int64_t D, int64_t
 template <int CB, int MODE>
 __global__ void __launch_bounds__(512, 1)
     cheb_step_f32_kernel(int nx, int ny, int64_t D, int64_t ldv, int ylen, const float2* __restrict__ table,
-                         const float4* __restrict__ Vcur, const float4* Vprev, float4* Vout, ColMap cmap,
+                         const float4* __restrict__ Vcur, const float4* Vprev, float4* Vout, int64_t s0,
                          double2* __restrict__ acc, const double* __restrict__ am, const double* __restrict__ ao,
                          int m) {
-  f32_step_body<CB, MODE>(nx, ny, D, ldv, ylen, table, Vcur, Vprev, Vout, cmap, acc, am, ao, m);
+  f32_step_body<CB, MODE>(nx, ny, D, ldv, ylen, table, Vcur, Vprev, Vout, s0, acc, am, ao, m);
 }
 
 // ---- TMA copies and bounded waits (the march kernel) ----------------------
@@ -1308,11 +1301,11 @@ cudaError_t launch_f32(const ChebPlan& p, const void* table, const void* Vcur, c
   if (mode == 0)
     cheb_step_f32_kernel<CB, 0><<<grid, p.nthreads, p.smem, s>>>(p.nx, p.ny, p.D, p.ldv, p.ylen, (const float2*)table,
                                                                  (const float4*)Vcur, (const float4*)Vprev, (float4*)Vout,
-                                                                 colmap(p, s0), acc, am, ao, m);
+                                                                 s0, acc, am, ao, m);
   else
     cheb_step_f32_kernel<CB, 1><<<grid, p.nthreads, p.smem, s>>>(p.nx, p.ny, p.D, p.ldv, p.ylen, (const float2*)table,
                                                                  (const float4*)Vcur, (const float4*)Vprev, (float4*)Vout,
-                                                                 colmap(p, s0), acc, am, ao, m);
+                                                                 s0, acc, am, ao, m);
   return cudaGetLastError();
 }
 template <int CB>

@@ -100,8 +100,9 @@ extern "C" int kpm_observables_noalloc(const kpm_model* m, const kpm_opts* o, co
   const size_t off_red = align256(off_ao + (size_t)o->M * sizeof(double));
   const size_t off_tab = align256(off_red + (size_t)reduce_scratch_doubles(0) * sizeof(double));
   // widest slab (unit columns per recursion) whose two buffers fit the rest: by the
-  // march kernel, or, where its chunk does not fit, by the narrower chunks of the
-  // one-step kernels
+  // march kernel, or, where one of its chunks (16 columns in FP32, 8 in FP64) does not fit, by the
+  // one-step kernels, whose chunks are narrower on rows of more than 122 (FP32) or 98 (FP64)
+  // sites and where cols_per_block asks for it (224x224 in FP32 runs 4 columns)
   size_t off_acc = 0, off_slab = 0;
   ChebPlan p;
   int64_t width = 0;
