@@ -1282,7 +1282,7 @@ int kpm_ldos(kpm_ctx* ctx, const kpm_model* model, const kpm_opts* opts, const d
   const int64_t D = 2 * (int64_t)N;
   const int M = opts->M;
   kpm_opts o = *opts;
-  o.flags &= ~KPM_FLAG_DOUBLE_STEP;  // one step per launch
+  o.flags &= ~KPM_FLAG_DOUBLE_STEP;  // the default steps per launch: two of unit vectors above L2
   if ((r = ensure_site_scratch(ctx, N))) return r;
   // scratch: record M x D, coefficients 2 x n_omega x M, weights 2N, frequencies n_omega
   const size_t rec_n = (size_t)M * D, c_n = 2 * (size_t)n_omega * M;
