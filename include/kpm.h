@@ -80,8 +80,12 @@ typedef struct {
                            kpm_observables_noalloc) */
   int32_t block_width;  /* unit start vectors per slab; 0 = as many as fit the
                            context's scratch budget (kpm_set_scratch_budget) */
-  int32_t cols_per_block; /* columns per CTA in the recursion kernel; 0 = default (FP32 unit
-                           vectors: always 16) */
+  int32_t cols_per_block; /* most columns per CTA of the one-step recursion kernels (FP64 and
+                           double-float probing, and kpm_observables_noalloc where the march
+                           kernel's columns do not fit); 0 = the most that fit.  Every other
+                           pass runs the march kernel, with 16 columns per CTA in FP32 and 8 in
+                           FP64 and double-float whatever is given here (narrower chunks were
+                           the slower the narrower they are); negative: KPM_EINVAL */
   double margin;        /* spectral half-width margin of the Gershgorin rescale (0.01) */
   double temperature;   /* 0: T = 0 step and min(eps, 0) in closed form; T > 0: Fermi
                            function 1/(1 + e^{eps/T}) and grand-potential function
@@ -105,13 +109,13 @@ typedef struct {
                            sites sum to the full pass exactly and the omegas to rounding.
                            kpm_observables and kpm_backward (its gradient is then the part
                            from those columns); with probing, KPM_EINVAL. */
-  int32_t band_rows;    /* lattice rows per CTA of the one-step recursion kernels (each
-                           CTA runs a band of rows of one column chunk); 0 = the
-                           library's choice (the best of a wave model: chunks x
-                           bands CTAs, one per SM, each costing its rows plus
-                           two halo rows of one vector), else min(band_rows, ny).  Changes the
-                           launch shape only, not the result; kpm_autotune searches
-                           it.  Negative: KPM_EINVAL. */
+  int32_t band_rows;    /* lattice rows per CTA of the recursion kernels (each CTA runs a
+                           band of rows of one column chunk, and of one tile of sites where a
+                           row takes several); 0 = the library's choice (the best of a
+                           wave model: the bands' CTAs run as many at a time as the SMs
+                           hold, each costing its rows and a start), else
+                           min(band_rows, ny).  Changes the launch shape only, not the
+                           result; kpm_autotune searches it.  Negative: KPM_EINVAL. */
 } kpm_opts;
 
 /* kpm_opts.flags: run the FP32 recursion on unit vectors one step more per
@@ -296,11 +300,11 @@ int rmft_update(kpm_ctx* ctx, const kpm_model* model, const kpm_rmft_opts* ropts
 
 /* Autotuner of the recursion launch: times two short passes (M = 18 and 34)
  * for every slab width in {D, 8192, ..., 128} (narrow slabs keep both
- * recursion vectors in L2), every column chunk that fits shared memory and
- * (FP32) the default steps per launch or one more, and for the default the
+ * recursion vectors in L2), every column chunk (the one-step kernels have
+ * several) and (FP32) the default steps per launch or one more, and for the default the
  * three best band heights of a wave model of the launch (CTAs of
- * ceil(ny / bands) rows, one per SM; the first is the default of band_rows
- * = 0) and one band per column chunk, predicts the pass at opts->M from the
+ * ceil(ny / bands) rows, as many at a time as the SMs hold; the first is the
+ * default of band_rows = 0) and one band per column chunk, predicts the pass at opts->M from the
  * line through both times (per-slab start and gather plus M - 1 steps), and
  * writes the fastest (block_width, cols_per_block, band_rows,
  * KPM_FLAG_DOUBLE_STEP bit of flags) into *best (other fields copied from
