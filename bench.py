@@ -640,7 +640,8 @@ def batched_section(kpm, inputs, torch, alu=None, iters=3):
     if rec_s > 0:
         # 106 flops per row-column (13 complex multiply-adds, one subtraction)
         tflops = 106.0 * row_updates / rec_s / 1e12
-        out["persistent_recursion"] = {
+        # the persistent launch of the small cells and the march kernel's of the others
+        out["recursion"] = {
             "s_per_iteration": rec_s, "launches_per_iteration": bst[0].recursion_launches,
             "effective_gbs": 24.0 * row_updates / rec_s / 1e9,
             "effective_note": "24 B per row-column (read V_m, V_m-1, write V_m+1) as if streamed; the vectors stay "
@@ -1086,11 +1087,11 @@ def profile_batched():
 
 def profile_small(double_step=False, precision="fp32"):
     """Small case for ncu: the benchmark lattice, slabs of 2000 columns
-    (2 x 320 MB, larger than L2), M = 8: seven recursion-step launches per
-    slab, in bands of 34 lattice rows (the band height the autotuner picks for
-    the benchmark's 20000-column slab, so that a launch reads the same halo
-    rows per column).  precision fp64 / df64: the same slabs through the FP64
-    or the double-float recursion."""
+    (320 MB each, larger than L2), M = 8.  FP32: three launches of two steps per
+    slab and one of one step, in one band of 100 lattice rows (the library's choice for the
+    benchmark's 20000-column slab, so that a launch reads the same halo rows per
+    column).  precision fp64 / df64: the same slabs through the FP64 or the
+    double-float recursion, seven launches of one step."""
     import torch
     from paper_2212_05685_gb300 import build, inputs, kpm
     build.build()
@@ -1107,7 +1108,7 @@ def profile_small(double_step=False, precision="fp32"):
     kpm.kpm_build_H(ctx, model, phi, params, 0.0, fields)
     kpm.kpm_bounds(ctx, model, fields, 0.01, ab)
     prec = {"fp32": kpm.KPM_FP32, "fp64": kpm.KPM_FP64, "df64": kpm.KPM_DF64}[precision]
-    kpm.kpm_observables(ctx, model, kpm.make_opts(8, prec, 2000, band_rows=34,
+    kpm.kpm_observables(ctx, model, kpm.make_opts(8, prec, 2000, band_rows=100,
                                                   flags=kpm.KPM_FLAG_DOUBLE_STEP if double_step else 0), fields, ab, obs)
     torch.cuda.synchronize()
     assert bool(torch.isfinite(obs).all())
