@@ -1366,14 +1366,16 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   // Between 640 and 720 Nambu rows it is the shape that decides (24 cells, M = 128): bands of
   // one row of up to 46 sites or two of up to 28 are the fastest persistent ones (21x16 7.07 / 7.70,
   // 22x16 7.38 / 7.74, 28x12 7.27 / 7.65, 41x8 7.42 / 7.66, 24x14 7.12 / 7.06), and narrow lattices the
-  // slowest on the march kernel (5x72 8.99 / 9.64, 7x48 7.88 / 8.40, 10x34 8.07 / 8.60, 8x41 7.69 / 7.41);
+  // slowest on the march kernel (5x72 8.99 / 9.64, 7x48 7.88 / 8.40, 10x34 8.07 / 8.60), but for 8 sites,
+  // whose rows fill its warps (8x41 7.69 / 7.41), and 7 in bands of seven rows (7x51 4% slower persistent);
   // the others are faster there (17x19 8.19 / 7.65, 13x26 8.22 / 7.93, 33x10 7.89 / 7.61).
   // Larger cells run the march kernel one after the other, over one pair of slabs, unless
   // the slabs do not fit the budget or the device; their launches go between two graphs
   // (a graph of them has cells x parts x M nodes).
   auto persist_rows = [](int nx, int ny) -> int64_t {
     const int band = (ny + 7) / 8;  // lattice rows of a CTA of the cluster
-    return nx <= 11 ? 720 : nx <= (band == 1 ? 46 : band == 2 ? 28 : 0) ? 704 : 640;
+    if (nx <= 11) return nx == 8 ? 640 : nx == 7 ? 672 : 720;
+    return nx <= (band == 1 ? 46 : band == 2 ? 28 : 0) ? 704 : 640;
   };
   std::vector<char> persist(members.size(), 0);
   size_t psmem = 0, march_slab = 0;

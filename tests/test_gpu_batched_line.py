@@ -1,6 +1,6 @@
 """The line between the persistent recursion and the march kernel in rmft_iterate_batched (FP32):
 640 Nambu rows, 704 where a CTA's band is one lattice row of up to 46 sites or two of up to 28, 720 up to
-11 sites wide.  On both sides of it the cells follow rmft_iterate (1e-12, as for the batch elsewhere);
+11 sites wide (7: 672, 8: 640).  On both sides of it the cells follow rmft_iterate (1e-12, as for the batch elsewhere);
 which route ran shows in the launches per iteration: one, or one a moment at least."""
 import pytest
 
@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,persistent", [
     (20, 16, True), (17, 19, False), (28, 12, True), (29, 12, False), (22, 16, True), (23, 16, False), (41, 8, True),
     (46, 7, True), (47, 7, False), (45, 8, False), (11, 30, True), (11, 33, False), (12, 27, False), (5, 72, True),
-    (5, 73, False), (50, 6, True), (33, 10, False)])
+    (5, 73, False), (8, 40, True), (8, 41, False), (7, 48, True), (7, 49, False), (9, 40, True), (50, 6, True), (33, 10, False)])
 def test_route_and_results_at_the_line(nx, ny, persistent):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
