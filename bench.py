@@ -594,7 +594,7 @@ def run_ours(args):
 
 def batched_section(kpm, inputs, torch, alu=None, iters=3):
     """32 cells of uneven size and doping (shapes 24x12 .. 64x32), M = 1024,
-    FP32: the batched call (cells of up to 640 Nambu rows in one persistent launch,
+    FP32: the batched call (small cells in one persistent launch,
     the others on the march kernel) vs the cells one after another; roofline of
     the batch's recursions against the measured FP32 FMA rate."""
     cells = inputs.cfg3_cells(seed=0, count=32)
