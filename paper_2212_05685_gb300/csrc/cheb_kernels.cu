@@ -1381,6 +1381,13 @@ cudaError_t march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, con
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  // FP64 rows are bound by the SM's FP64 pipe.  Launched while the grid before finishes, CTAs
+  // went two to an SM that was free where others were about to be: with no more CTAs than SMs,
+  // each takes more than half of the shared memory, so that they stay apart.  us a step: 24x4
+  // 12.8 -> 7.6, 20x5 11.0 -> 7.3, 9x8 10.3 -> 6.2, 8x8 8.4 -> 6.1 (one-step kernel 10.9, 9.1, 8.8, 8.8).
+  // (Not in graphs, where they spread by themselves and cells of a batch run side by side.)
+  if (EL == kElF64 && cfg.numAttrs == 1 && (int64_t)grid.x * grid.y <= kSMs)
+    cfg.dynamicSmemBytes = std::max<size_t>(mp.smem, 116 * 1024);
   return cudaLaunchKernelEx(&cfg, fn, v, pr, a, cm);
 }
 }  // namespace
