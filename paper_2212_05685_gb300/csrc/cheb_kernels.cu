@@ -1394,16 +1394,18 @@ cudaError_t march_launch(const MarchPlan& mp, dim3 grid, const MarchMaps& v, con
 
 namespace {
 // band heights of a march launch: as many CTAs per SM as registers and shared memory
-// take; a CTA's start (barriers, first copies) costs about five rows (one of double-float;
-// 0.3 of FP64, whose rows are bound by the FP64 pipe: passes of M = 65 with 1.0 and 0.3, ms:
-// 40x11 5.71 and 4.97, 45x10 6.21 and 5.43, 30x21 11.71 and 10.61, 104x7 14.33 and 13.27),
-// and a launch of several steps computes two more rows for every step but the last
+// take; a CTA's start (barriers, first copies) costs about five rows (one of double-float),
+// and a launch of several steps computes two more rows for every step but the last.
+// FP64 rows are bound by the FP64 pipe and long: a start is 0.4 of one (passes of M = 65 with 1.0
+// and 0.4, ms: 40x11 5.72 and 4.97, 45x10 6.22 and 5.43, 30x21 11.7 and 10.6, 104x7 14.3 and 13.3).
+// Beside the launches of other streams the fewer, higher bands of 1.0 leave room for them:
+// batches of 40x11, 45x10, 30x21 cells 18.1 and 19.4 ms, of 45x10 and 36x20 33.2 and 34.2.
 int march_per_sm(const MarchPlan& p) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(16 / p.warps, (int64_t)(228 * 1024) / (int64_t)(p.smem + 1024)));
 }
 int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
   const int per_sm = march_per_sm(p);
-  const double start = p.el == kElF32 ? 5.0 + 2.0 * (p.ns - 1) : p.el == kElDF ? 1.0 : 0.3;
+  const double start = p.el == kElF32 ? 5.0 + 2.0 * (p.ns - 1) : p.el == kElDF || p.beside ? 1.0 : 0.4;
   return band_rows_candidates(ny, ldv / march_cols(p.el) * p.ntile, out, maxn, per_sm * kSMs, start);
 }
 
@@ -1412,9 +1414,10 @@ int march_bands(const MarchPlan& p, int ny, int64_t ldv, int* out, int maxn) {
 // memory (several steps: eight rows each), and the band height of the wave model.
 // (Two steps in tiles of 26 sites do not fit: 104x104 in five tiles of 21, M = 65, 96.6 ms, one
 // step 113.2; 180x60 in eight of 23, M = 33, 53.0 and 56.3.)
-MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows, int el = kElF32) {
+MarchPlan plan_march(int nx, int ny, int64_t ldv, int ns, int band_rows, int el = kElF32, bool beside = false) {
   MarchPlan p;
   p.el = el;
+  p.beside = beside;
   constexpr int nv = kMarchLanes;
   auto warps = [&](int tx, bool full) {
     int n = 2;  // the producer and the moment sums
@@ -1557,7 +1560,7 @@ int band_rows_candidates(int ny, int64_t ctas, int* out, int maxn, int slots, do
 }
 
 ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request, int band_rows, int steps,
-                   bool split) {
+                   bool split, bool beside) {
   ChebPlan p;
   p.nx = nx;
   p.ny = ny;
@@ -1605,7 +1608,7 @@ ChebPlan plan_cheb(int nx, int ny, int64_t width, int precision, int cb_request,
     p.cb = march_cols(el);
     p.ldv = (width + p.cb - 1) / p.cb * p.cb;
     p.sub = split && steps == 1 && el == kElF32 ? march_columns(nx, ny, p.ldv) : p.ldv;
-    p.m1 = plan_march(nx, ny, p.sub, 1, band_rows, el);
+    p.m1 = plan_march(nx, ny, p.sub, 1, band_rows, el, beside);
     p.mk = steps > 1 && el == kElF32 ? plan_march(nx, ny, p.ldv, steps, band_rows) : p.m1;
     if (p.mk.ns == 0) p.mk = p.m1;
     p.ylen = p.mk.ylen;

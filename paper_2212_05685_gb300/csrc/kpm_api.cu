@@ -1353,7 +1353,7 @@ int rmft_iterate_batched(kpm_ctx* ctx, int ncell, const kpm_model* models, const
   for (size_t k = 0; k < members.size(); ++k) {
     const kpm_model& m0 = models[members[k][0]];
     const int64_t D = 2 * (int64_t)m0.nx * m0.ny;
-    plans[k] = plan_cheb(m0.nx, m0.ny, D, prec, opts->cols_per_block, opts->band_rows, 1, true);
+    plans[k] = plan_cheb(m0.nx, m0.ny, D, prec, opts->cols_per_block, opts->band_rows, 1, true, members.size() > 1);
     if (plans[k].cb == 0) return fail(ctx, KPM_EINVAL, "lattice row too wide for the shared-memory window");
     cudaError_t e = cheb_prepare(plans[k], prec);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "prepare");

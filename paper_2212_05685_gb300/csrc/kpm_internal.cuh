@@ -18,6 +18,7 @@ constexpr int kRedBlock = 256; // threads of the reduction kernels
 struct MarchPlan {
   int ns = 0;                  // steps per launch (0: not planned)
   int el = 0;                  // element: 0 FP32 column pairs, 1 double-float, 2 FP64
+  bool beside = false;         // launched beside other streams' launches
   int tx = 0, ntile = 0, full = 0;  // sites per tile, tiles per lattice row, one tile covers the row
   int ylen = 0;                // lattice rows per band
   int wrow = 0, crowb = 0;     // sites of a ring row, bytes of its entries
@@ -129,9 +130,10 @@ int reduce_scratch_doubles(int64_t n);
 // ---------------------------------------------------------------- cheb_kernels.cu
 // steps: recursion steps per launch of the march kernel (FP64 and double-float: one;
 // chunks of 16 FP32 columns or 8); 0: the one-step kernels with their narrower chunks.
-// split: FP32 single steps over parts of the slab (march_columns)
+// split: FP32 single steps over parts of the slab (march_columns).
+// beside: the launches share the device with those of other streams
 ChebPlan plan_cheb(int nx, int ny, int64_t ldv_cols, int precision, int cb_request, int band_rows = 0, int steps = 0,
-                   bool split = false);
+                   bool split = false, bool beside = false);
 // FP32 steps per launch at which unit-vector slabs of `width` columns run fastest
 int march_steps(int nx, int ny, int64_t width);
 // and the columns of a slab of `width` that run all their single steps before the next ones
